@@ -48,4 +48,21 @@ __device__ __forceinline__ int corr_entry(const DevProblem& pb, const uint32_t* 
     return (int)cidx[c] + sf * pb.site_w[ent];
 }
 
+// lane-serial version used while every lane evaluates its own hop
+template <typename R>
+__device__ R corr_ratio_serial(const DevProblem& pb, const uint32_t* cidx, int p, int q) {
+    int ns = pb.ns;
+    int sf = p >= ns ? 2 : 1;
+    int sp = p >= ns ? p - ns : p, sq = q >= ns ? q - ns : q;
+    int total = (pb.site_cptr[sp + 1] - pb.site_cptr[sp]) + (pb.site_cptr[sq + 1] - pb.site_cptr[sq]);
+    R prod = R(1);
+#pragma unroll 4
+    for (int e = 0; e < total; ++e) {
+        int c;
+        int newi = corr_entry(pb, cidx, sp, sq, sf, e, &c);
+        if (c >= 0) prod *= load_C<R>(pb, pb.corr_off[c] + newi) / load_C<R>(pb, pb.corr_off[c] + cidx[c]);
+    }
+    return prod;
+}
+
 }  // namespace vmc

@@ -49,10 +49,6 @@ struct vmc_ctx {
     int maxd = 1;
     int max_csites = 0;          // sites of the largest correlator
     bool ff_sums = true;         // FP32-store passes with FP64 sums in FP32-pair arithmetic
-    // shared-memory carveout of the FP32 ab initio walkers in percent: 58 (two
-    // 4-walker CTAs per SM, more L1 for the tables) measured 213 ms against
-    // 221 ms at the driver's choice and 333 ms at 30 (24 orbitals, 65,536 samples)
-    int walker_carveout_ab = 58;
     bool params_set = false, walkers_set = false;
     bool use_stream = true;     // TMA-staged pass for FP32-accumulation products
     bool stream_cached = false;  // register-cached variant for BF16, one vector (slower: 16 warps)
@@ -107,7 +103,8 @@ struct vmc_ctx {
     float *d_h32 = nullptr, *d_eri32 = nullptr;
     int *d_pair_ptr = nullptr, *d_pair_corr = nullptr;
     uint16_t* d_dexc = nullptr;   // double-excitation pair tables (ab initio)
-    bool pair_unique = false;     // no site pair lies in two correlators (and ncp < 2^30)
+    double* d_erijk64 = nullptr;  // Coulomb and exchange rows of eri
+    float* d_erijk32 = nullptr;
     double *d_C64 = nullptr, *d_invC64 = nullptr, *d_F64 = nullptr;
     float *d_C32 = nullptr, *d_invC32 = nullptr, *d_F32 = nullptr;
     uint16_t* d_pairtab = nullptr;
@@ -132,6 +129,9 @@ struct vmc_ctx {
     unsigned char* d_batch = nullptr;   // argument blocks of batched launches led by this handle
     size_t batch_bytes = 0;
     double* d_pf64 = nullptr;
+    char* d_abX = nullptr;       // ab initio: [ncap][N][N] pairing inverses for the local energy's pass
+    size_t abX_bytes = 0;
+    uint8_t* d_abpos = nullptr;  // [ncap][Nst] the orbitals at their positions
     float* d_pf32 = nullptr;
     __nv_bfloat16* d_pf16 = nullptr;
     double* d_Obar[3] = {nullptr, nullptr, nullptr};
@@ -353,11 +353,9 @@ extern "C" int vmc_create(const vmc_lattice* lat, const vmc_hamiltonian* ham, co
             for (int j1 = cptr[c]; j1 < cptr[c + 1]; ++j1)
                 for (int j2 = cptr[c]; j2 < cptr[c + 1]; ++j2)
                     if (j1 != j2) pl[(size_t)csites[j1] * ns + csites[j2]].push_back(c);
-        h->pair_unique = h->ncp < ((int64_t)1 << 30);
         for (size_t k = 0; k < pl.size(); ++k) {
             for (int c : pl[k]) pcorr.push_back(c);
             pptr[k + 1] = (int)pcorr.size();
-            if (pl[k].size() > 1) h->pair_unique = false;
         }
     }
     // ab initio integrals: (pq|rs) = sum_mu L^mu_pq L^mu_rs (Eq. 9 with R = L)
@@ -492,6 +490,23 @@ extern "C" int vmc_create(const vmc_lattice* lat, const vmc_hamiltonian* ham, co
         UPL(h->d_h32, h32.data(), h32.size());
         UPL(h->d_eri64, eri64.data(), eri64.size());
         UPL(h->d_eri32, eri32.data(), eri32.size());
+        {
+            const size_t nk = (size_t)round_up(ns, 4), nt = (size_t)ns * ns;
+            std::vector<double> jk(nt * 2 * nk, 0.0);
+            for (int p = 0; p < ns; ++p)
+                for (int q = 0; q < ns; ++q) {
+                    double* row = jk.data() + 2 * nk * ((size_t)p * ns + q);
+                    for (int k = 0; k < ns; ++k) {
+                        row[k] = eri64[(((size_t)p * ns + q) * ns + k) * ns + k];
+                        row[nk + k] = eri64[(((size_t)p * ns + k) * ns + k) * ns + q];
+                    }
+                }
+            std::vector<float> jk32(jk.begin(), jk.end());
+            ACK(h->alloc(&h->d_erijk64, jk.size()));
+            ACK(h->alloc(&h->d_erijk32, jk32.size()));
+            UPL(h->d_erijk64, jk.data(), jk.size());
+            UPL(h->d_erijk32, jk32.data(), jk32.size());
+        }
         // double excitations: electron-position pairs, then empty-orbital
         // index pairs, of the up-up, down-down and up-down classes
         const int eu = ns - nu, ed = ns - nd;
@@ -625,7 +640,8 @@ extern "C" int vmc_create(const vmc_lattice* lat, const vmc_hamiltonian* ham, co
     pb.nbr_ptr = h->d_nbr_ptr; pb.nbr_site = h->d_nbr_site; pb.nbr_t = h->d_nbr_t;
     pb.h64 = h->d_h64; pb.h32 = h->d_h32; pb.eri64 = h->d_eri64; pb.eri32 = h->d_eri32;
     pb.pair_ptr = h->d_pair_ptr; pb.pair_corr = h->d_pair_corr;
-    pb.pair_unique = h->pair_unique ? 1 : 0;
+    pb.erijk64 = h->d_erijk64; pb.erijk32 = h->d_erijk32;
+    pb.eri_nk = (int)round_up(ns, 4);
     pb.dexc = h->d_dexc;
     pb.max_csites = h->max_csites;
     pb.ff_sums = h->ff_sums ? 1 : 0;
@@ -765,19 +781,10 @@ static int read_status(vmc_ctx* h, cudaStream_t st) {
 static size_t prep_walkers(vmc_ctx* h, SampleArgs& a, bool fp64) {
     a.pb = h->pb;
     a.XS = (h->N + 2) & ~1;   // even (the rank-2 update moves column pairs), N + 1 or N + 2
-    a.GS = h->N + 1;
     a.ncorr_pad = (int)round_up(std::max(h->ncorr, 1), 4);
     const size_t rsz = fp64 ? 8 : 4;
     size_t wb = (size_t)h->N * a.XS * rsz + 3 * (size_t)a.XS * rsz;
     wb = wb + 64 + (size_t)a.ncorr_pad * 4 + 64 + 128;
-    if (h->ham == VMC_ABINITIO && a.want_energy) {
-        // G [M][GS], H [E][E], single-move factors [N][E], empty list, index
-        // map, per-site factors [ns][4]
-        const size_t E = (size_t)(h->M - h->N);
-        wb += ((size_t)h->M * a.GS + E * E + (size_t)h->N * E) * rsz + 128 + 128 + (size_t)4 * h->ns * rsz;
-        // the sample's site-pair table (pair correlators, each pair in at most one)
-        if (h->max_csites <= 2 && h->pair_unique) wb += (size_t)h->ns * (h->ns - 1) / 2 * 4;
-    }
     wb = round_up(wb, 16);
     a.warp_bytes = wb;
     a.status = h->d_status;
@@ -790,22 +797,15 @@ static int launch_walkers(vmc_ctx* h, SampleArgs& a, bool fp64, cudaStream_t st)
     if (wpb < 1) return VMC_ERR_UNSUPPORTED;
     size_t smem = wb * wpb;
     int blocks = (a.n_walkers + wpb - 1) / wpb;
-    if (fp64) {
-        VCK(cudaFuncSetAttribute(k_walkers<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_walkers<double><<<blocks, 32 * wpb, smem, st>>>(a); h->n_launch++;
-    } else {
-        VCK(cudaFuncSetAttribute(k_walkers<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        // shared-memory carveout (percent of the maximum): the ab initio local
-        // energy reads integral, correlator and pair tables through L1
-        VCK(cudaFuncSetAttribute(k_walkers<float>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 h->ham == VMC_ABINITIO ? h->walker_carveout_ab : -1));
-        k_walkers<float><<<blocks, 32 * wpb, smem, st>>>(a); h->n_launch++;
-    }
+    auto kern = fp64 ? k_walkers<double> : k_walkers<float>;
+    VCK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kern<<<blocks, 32 * wpb, smem, st>>>(a); h->n_launch++;
     VCK(cudaGetLastError());
     return VMC_OK;
 }
 
-static void store_targets(vmc_ctx* h, SampleArgs& a) {
+// where walkers of the given precision write the O store
+static int store_targets(vmc_ctx* h, SampleArgs& a, bool fp64) {
     a.s_occ = h->d_socc; a.Nst = h->Nst;
     a.s_cidx = h->d_cidx; a.ncst = h->ncst;
     a.s_E = h->d_E;
@@ -814,6 +814,62 @@ static void store_targets(vmc_ctx* h, SampleArgs& a) {
     a.s_pf32 = h->keeplow ? h->d_pf32 : nullptr;
     a.s_pf16 = h->keeplow ? h->d_pf16 : nullptr;
     a.Pst = h->Pst;
+    if (h->ham == VMC_ABINITIO) {
+        // what the local energy's pass reads (FP64 walkers and refreshes: twice the bytes)
+        const size_t bytes = (size_t)h->ncap * h->N * h->N * (fp64 ? 8 : 4);
+        if (h->abX_bytes < bytes) {
+            if (h->d_abX) {
+                VCK(cudaFree(h->d_abX));   // waits for the work that reads it
+                h->allocs.erase(std::find(h->allocs.begin(), h->allocs.end(), (void*)h->d_abX));
+                h->d_abX = nullptr;
+                h->abX_bytes = 0;
+            }
+            VCK(h->alloc(&h->d_abX, bytes));
+            h->abX_bytes = bytes;
+        }
+        if (!h->d_abpos) VCK(h->alloc(&h->d_abpos, (size_t)h->ncap * h->Nst));
+        a.s_X = h->d_abX;
+        a.s_pos = h->d_abpos;
+    }
+    return VMC_OK;
+}
+
+// E_L of the stored samples of an ab initio problem, from the pairing inverses
+// that walkers of the given precision wrote (the Hubbard energy is the
+// walkers' own).  Four warps per sample; two or one where the tables of a
+// large FP64 problem leave no room for more, and the general correlator
+// factors where they do not fit at all or correlators span more sites.
+static int ab_energy(vmc_ctx* h, bool fp64, int64_t n_s, cudaStream_t st) {
+    if (h->ham != VMC_ABINITIO || n_s == 0) return VMC_OK;
+    const size_t rsz = fp64 ? 8 : 4;
+    AbArgs a{};
+    a.pb = h->pb;
+    a.n_s = n_s;
+    a.pos = h->d_abpos; a.Nst = h->Nst;
+    a.s_cidx = h->d_cidx; a.ncst = h->ncst;
+    a.X = h->d_abX;
+    a.s_E = h->d_E;
+    a.status = h->d_status;
+    const size_t rest = (size_t)h->N * (h->N | 1) * rsz + (size_t)h->ncorr * 4 + 64 + 3 * 128;
+    int nw = kAbThreads / 32;
+    AbLayout L = ab_layout(h->ns, h->nu, h->nd, nw);
+    if (h->max_csites <= 2) {
+        while (nw > 1 && round_up(L.n, 4) * rsz + rest + 64 > h->smem_optin) {
+            nw /= 2;
+            L = ab_layout(h->ns, h->nu, h->nd, nw);
+        }
+        a.pairs = round_up(L.n, 4) * rsz + rest + 64 <= h->smem_optin;
+    }
+    if (!a.pairs) {
+        nw = kAbThreads / 32;
+        L = ab_layout(h->ns, h->nu, h->nd, nw);
+    }
+    a.elems = (int)round_up(a.pairs ? L.n : L.g0 + h->N * (h->M - h->N), 4);
+    const size_t smem = a.elems * rsz + rest;
+    if (smem + 64 > h->smem_optin) return VMC_ERR_UNSUPPORTED;
+    VCK(launch_ab_energy(fp64, a, 32 * nw, smem, h->nsm, st));
+    h->n_launch++;
+    return VMC_OK;
 }
 
 static int transpose_states(vmc_ctx* h, cudaStream_t st) {
@@ -824,7 +880,7 @@ static int transpose_states(vmc_ctx* h, cudaStream_t st) {
     return VMC_OK;
 }
 
-static void sample_args(vmc_ctx* h, int n_burn, uint64_t seed, SampleArgs& a) {
+static int sample_args(vmc_ctx* h, int n_burn, uint64_t seed, SampleArgs& a) {
     a = SampleArgs{};
     a.n_walkers = h->n_walkers;
     a.spw = h->spw;
@@ -836,7 +892,7 @@ static void sample_args(vmc_ctx* h, int n_burn, uint64_t seed, SampleArgs& a) {
     a.seed = seed;
     a.walker_occ = h->d_wocc;
     a.walker_step = h->d_wstep;
-    store_targets(h, a);
+    return store_targets(h, a, h->wprec == VMC_FP64);
 }
 
 static int after_sampling(vmc_ctx* h, cudaStream_t st);
@@ -846,20 +902,24 @@ extern "C" int vmc_sample(vmc_handle h, int n_burn, uint64_t seed, void* stream)
     if (!h->params_set || !h->walkers_set) return VMC_ERR_STATE;
     cudaStream_t st = (cudaStream_t)stream;
     SampleArgs a;
-    sample_args(h, n_burn, seed, a);
-    int rc = launch_walkers(h, a, h->wprec == VMC_FP64, st);
+    int rc = sample_args(h, n_burn, seed, a);
+    if (rc) return rc;
+    rc = launch_walkers(h, a, h->wprec == VMC_FP64, st);
     if (rc) return rc;
     return after_sampling(h, st);
 }
 
 // the store holds a new set of samples: invalidate what was built on the old
-// one, refresh in FP64 if asked, transpose the correlator states
+// one, the ab initio energies, refresh in FP64 if asked, transpose the
+// correlator states
 static int after_sampling(vmc_ctx* h, cudaStream_t st) {
     int rc;
     h->n_s = h->ncap;
     h->obar_ok[0] = h->obar_ok[1] = h->obar_ok[2] = false;
     h->sorted_ok = h->g_ok = h->corr_ok = false;
     h->refreshed = false;
+    rc = ab_energy(h, h->wprec == VMC_FP64, h->n_s, st);
+    if (rc) return rc;
     if (h->wprec == VMC_FP32 && h->fp64_refresh) {
         // FP64 refresh of every stored sample: the pairing inverse, E_L and O
         // from scratch in FP64, rounded into the stores; the chains' own E_L
@@ -871,9 +931,11 @@ static int after_sampling(vmc_ctx* h, cudaStream_t st) {
         m.spw = 1;
         m.want_energy = 1;
         m.walker_occ = h->d_mocc;
-        store_targets(h, m);
+        rc = store_targets(h, m, true);
+        if (rc) return rc;
         m.s_lnrun = nullptr;   // keep the chains' running log-amplitudes
         rc = launch_walkers(h, m, true, st);
+        if (!rc) rc = ab_energy(h, true, h->n_s, st);
         if (rc) return rc;
         h->refreshed = true;
     }
@@ -915,7 +977,8 @@ extern "C" int vmc_sample_batch(const vmc_handle* hs, int n, int n_burn, const u
     std::vector<int> wstart(n + 1, 0);
     size_t wb = 0;
     for (int b = 0; b < n; ++b) {
-        sample_args(hs[b], n_burn, seeds[b], args[b]);
+        int rs = sample_args(hs[b], n_burn, seeds[b], args[b]);
+        if (rs) return rs;
         wb = std::max(wb, prep_walkers(hs[b], args[b], fp64));
         wstart[b + 1] = wstart[b] + hs[b]->n_walkers;
     }
@@ -954,10 +1017,12 @@ static int measure_device_configs(vmc_ctx* h, int64_t n_s, bool fp64, const doub
     a.want_energy = bgrad ? 0 : 1;
     a.walker_occ = h->d_mocc;
     a.walker_step = nullptr;
-    if (to_store) store_targets(h, a);
+    int rc = to_store ? store_targets(h, a, fp64) : VMC_OK;
+    if (rc) return rc;
     a.bw = bw;
     a.bgrad = bgrad;
-    return launch_walkers(h, a, fp64, st);
+    rc = launch_walkers(h, a, fp64, st);
+    return rc || !to_store ? rc : ab_energy(h, fp64, n_s, st);
 }
 
 extern "C" int vmc_measure(vmc_handle h, const uint8_t* occ, int64_t n_s, void* stream) {

@@ -120,10 +120,14 @@ struct DevProblem {
     const float* h32;
     const double* eri64;
     const float* eri32;
+    // Coulomb and exchange rows (pq|kk) and (pk|kq), k < ns: [ns][ns][2][eri_nk],
+    // padded with zeros to eri_nk (a multiple of four)
+    const double* erijk64;
+    const float* erijk32;
+    int eri_nk;
     // correlators containing both sites i and j: pair_corr[pair_ptr[i ns + j] ..]
     const int* pair_ptr;
     const int* pair_corr;
-    int pair_unique;           // no site pair lies in two correlators (and ncp < 2^30): per-sample pair table
     // double excitations: electron-position pairs (a | b << 8) of the up-up,
     // down-down and up-down classes, then empty-orbital index pairs (ix | iy << 8)
     // of the same classes (ab initio only)

@@ -23,7 +23,6 @@ struct SampleArgs {
     uint8_t* walker_occ;  // [n_walkers][N] ascending on entry
     uint64_t* walker_step;
     int XS;               // row stride of the inverse in shared memory
-    int GS;               // row stride of G (ab initio local energy)
     int ncorr_pad;
     size_t warp_bytes;
     // O store
@@ -37,11 +36,58 @@ struct SampleArgs {
     float* s_pf32;
     __nv_bfloat16* s_pf16;
     int64_t Pst;
+    void* s_X;            // [n_s][N][N] the pairing inverse in the walker's precision (may be null)
+    uint8_t* s_pos;       // [n_s][Nst] the orbitals at its positions
     // adjoint mode: bgrad[k] += bw[s] O_k(n_s) instead of writing the store
     const double* bw;
     double* bgrad;
     int* status;
 };
+
+// Shared-memory tables of the ab initio local energy of one sample (elements
+// of R from the start of the region; the Quad block stays 16-byte aligned).
+struct AbLayout {
+    int GS, evs;                // row stride of G; elements of a warp's ev block
+    int ev, G, H[3], g0, gss, g1, t2, s1, rup, rdn, n;
+};
+__host__ __device__ inline AbLayout ab_layout(int ns, int nu, int nd, int nw) {
+    AbLayout L;
+    const int N = nu + nd, E = 2 * ns - N, eu = ns - nu, ed = ns - nd;
+    L.GS = N | 1;
+    L.ev = 0;                                   // a Quad and a value per warp and site
+    L.evs = (5 * ns + 3) / 4 * 4;
+    L.G = L.ev + nw * L.evs;                       // G[hole][electron]
+    L.H[0] = L.G + E * L.GS;                    // [x][y], up-up
+    L.H[1] = L.H[0] + eu * eu;                  // [x][y], x up, y down
+    L.H[2] = L.H[1] + eu * ed;                  // [x][y], down-down
+    L.g0 = L.H[2] + ed * ed;                    // [t][s]
+    L.gss = L.g0 + ns * ns;                     // [t][s], one spin at a time
+    L.g1 = L.gss + ns * ns;                     // [up electron][up hole], then [up hole][up electron]
+    L.t2 = L.g1 + 2 * nu * eu;                    // [down electron][down hole][4]; rsite [ns][4] before it is built
+    const int t2 = 4 * nd * ed;
+    L.s1 = L.t2 + (t2 > 4 * ns ? t2 : 4 * ns);  // [a][x], one spin at a time
+    L.rup = L.s1 + (nu * eu > nd * ed ? nu * eu : nd * ed);
+    L.rdn = L.rup + ns;                         // [s][2]
+    L.n = L.rdn + 2 * ns;
+    return L;
+}
+
+// Ab initio local energy of the stored samples (abinitio.cu)
+constexpr int kAbThreads = 128;
+struct AbArgs {
+    DevProblem pb;
+    int64_t n_s;
+    const uint8_t* pos;     // [n_s][Nst] orbitals at the positions of X, up before down
+    int Nst;
+    const cstate_t* s_cidx;
+    int ncst;
+    const void* X;          // [n_s][N][N] the pairing inverse in the walkers' precision
+    int pairs;              // the tables of pair correlators (else the general correlator factors)
+    int elems;              // elements of the tables
+    double* s_E;
+    int* status;
+};
+cudaError_t launch_ab_energy(bool fp64, const AbArgs& a, int threads, size_t smem, int nsm, cudaStream_t st);
 
 struct LogPsiArgs {
     DevProblem pb;
@@ -55,7 +101,7 @@ struct LogPsiArgs {
     double* out;
 };
 
-template <typename R> __global__ void k_walkers(SampleArgs a);
+template <typename R> __global__ void __launch_bounds__(128, 4) k_walkers(SampleArgs a);
 cudaError_t launch_walkers_batch(bool fp64, int blocks, int threads, size_t smem, cudaStream_t st,
                                  const SampleArgs* args, const int* wstart, int n, size_t warp_bytes);
 __global__ void k_logpsi(LogPsiArgs a);
