@@ -48,7 +48,11 @@ struct vmc_ctx {
     int ham = 0;
     int maxd = 1;
     int max_csites = 0;          // sites of the largest correlator
-    bool ff_sums = true;         // FP32-store passes with FP64 sums in FP32-pair arithmetic
+    struct PassPlan {            // launch shape of a pass with FP64 sums (see plan_pass)
+        int ni = 0;              // images per CTA
+        int64_t n_s = -1;        // of the samples that it is for (-1: not planned)
+        size_t smem = 0;
+    } pass_plan[4];              // one, two, four vectors; the gradient
     bool params_set = false, walkers_set = false;
     bool use_stream = true;     // TMA-staged pass for FP32-accumulation products
     bool stream_cached = false;  // register-cached variant for BF16, one vector (slower: 16 warps)
@@ -548,6 +552,22 @@ extern "C" int vmc_create(const vmc_lattice* lat, const vmc_hamiltonian* ham, co
     ACK(h->alloc(&h->d_lnrun, h->ncap));
     if (h->fp64_refresh) ACK(h->alloc(&h->d_Echain, h->ncap));
     if (h->keep64) ACK(h->alloc(&h->d_pf64, (size_t)h->ncap * h->Pst));
+    {
+        std::vector<uint32_t> ft;
+        const int Puu = nu * (nu - 1) / 2, Pdd = nd * (nd - 1) / 2;
+        for (int a = 0; a < N; ++a)
+            for (int b = a + 1; b < N; ++b) {
+                int e;
+                if (b < nu) e = a * nu - a * (a + 1) / 2 + (b - a - 1);
+                else if (a >= nu) e = Puu + (a - nu) * nd - (a - nu) * (a - nu + 1) / 2 + (b - a - 1);
+                else e = Puu + Pdd + a * nd + (b - nu);
+                ft.push_back((uint32_t)e | ((uint32_t)a << 16) | ((uint32_t)b << 24));
+            }
+        ACK(h->alloc(&h->d_fulltab, std::max<size_t>(ft.size(), 1)));
+        if (!ft.empty() && cudaMemcpy(h->d_fulltab, ft.data(), sizeof(uint32_t) * ft.size(),
+                                      cudaMemcpyHostToDevice) != cudaSuccess)
+            return fail(VMC_ERR_CUDA);
+    }
     if (h->keeplow) {
         ACK(h->alloc(&h->d_pf32, (size_t)h->ncap * h->Pst));
         ACK(h->alloc(&h->d_pf16, (size_t)h->ncap * h->Pst));
@@ -558,20 +578,6 @@ extern "C" int vmc_create(const vmc_lattice* lat, const vmc_hamiltonian* ham, co
             const int QE = (h->P + kGParts - 1) / kGParts;
             h->gwq = (QE + 3) / 4;
             h->Gst = (int64_t)kGParts * h->gwq * 4;
-            std::vector<uint32_t> ft;
-            const int Puu = nu * (nu - 1) / 2, Pdd = nd * (nd - 1) / 2;
-            for (int a = 0; a < N; ++a)
-                for (int b = a + 1; b < N; ++b) {
-                    int e;
-                    if (b < nu) e = a * nu - a * (a + 1) / 2 + (b - a - 1);
-                    else if (a >= nu) e = Puu + (a - nu) * nd - (a - nu) * (a - nu + 1) / 2 + (b - a - 1);
-                    else e = Puu + Pdd + a * nd + (b - nu);
-                    ft.push_back((uint32_t)e | ((uint32_t)a << 16) | ((uint32_t)b << 24));
-                }
-            ACK(h->alloc(&h->d_fulltab, std::max<size_t>(ft.size(), 1)));
-            if (!ft.empty() && cudaMemcpy(h->d_fulltab, ft.data(), sizeof(uint32_t) * ft.size(),
-                                          cudaMemcpyHostToDevice) != cudaSuccess)
-                return fail(VMC_ERR_CUDA);
         }
         ACK(h->alloc(&h->d_G, (size_t)h->ncap * h->Gst));
         // compact copy: the values of each row in the row-major pair order,
@@ -644,7 +650,6 @@ extern "C" int vmc_create(const vmc_lattice* lat, const vmc_hamiltonian* ham, co
     pb.eri_nk = (int)round_up(ns, 4);
     pb.dexc = h->d_dexc;
     pb.max_csites = h->max_csites;
-    pb.ff_sums = h->ff_sums ? 1 : 0;
     pb.C64 = h->d_C64; pb.C32 = h->d_C32; pb.F64 = h->d_F64; pb.F32 = h->d_F32;
     pb.pairtab = h->d_pairtab; pb.rowbase = h->d_rowbase;
     *out = h;
@@ -1167,13 +1172,99 @@ extern "C" int vmc_logpsi_backward(vmc_handle h, const double* w, double* grad, 
 // ---------------------------------------------------------------------------
 // streaming passes over the O store
 // ---------------------------------------------------------------------------
-template <typename ST, typename AT, int K, bool G>
-static int launch_main(vmc_ctx* h, const void* s_pf, const AT* V, const AT* invC, AT* T, const int* stop,
+// launch shape of a pass with FP64 sums over K vectors (gather) or for the
+// gradient (t_s given, K = 2): as many images per CTA as shared memory holds,
+// up to one per warp
+static int plan_pass(vmc_ctx* h, int K, bool gather, vmc_ctx::PassPlan** out) {
+    vmc_ctx::PassPlan& L = h->pass_plan[!gather ? 3 : K == 1 ? 0 : K == 2 ? 1 : 2];
+    if (L.n_s != h->n_s) {
+        int ni = pass_warps(K);
+        while (ni > 1 && pass_smem(h->npf, h->P, K, gather, ni) > h->smem_optin) ni /= 2;
+        if (pass_smem(h->npf, h->P, K, gather, ni) > h->smem_optin) {
+            set_err("pairing block does not fit in shared memory");
+            return VMC_ERR_UNSUPPORTED;
+        }
+        // no more images than the samples of a CTA pay for: an image is cleared
+        // and added up once per element of the pairing block
+        const double per_cta = (double)h->n_s * h->P / h->nsm;
+        while (ni > 1 && (double)ni * h->npf > per_cta) ni /= 2;
+        L.smem = pass_smem(h->npf, h->P, K, gather, ni);
+        L.ni = ni;
+        L.n_s = h->n_s;
+    }
+    *out = &L;
+    return VMC_OK;
+}
+
+static void pass_args(const vmc_ctx* h, const vmc_ctx::PassPlan& L, int K, const void* s_pf, const double* V, double* T,
+                      const int* stop, PassArgs& a) {
+    a = PassArgs{};
+    a.pb = h->pb;
+    a.n_s = h->n_s;
+    a.s_occ = h->d_socc; a.Nst = h->Nst;
+    a.s_cidx = h->d_cidx; a.ncst = h->ncst;
+    a.s_pf = s_pf; a.Pst = h->Pst;
+    a.fulltab = h->d_fulltab;
+    a.V = V; a.invC = h->d_invC64; a.T = T;
+    a.pf_partial = (double*)h->d_pfpart;
+    a.ni = L.ni;
+    a.stop = stop;
+    // orbitals where an image's owners begin: equal shares of the expected number
+    // of pairs (p, q > p) at the sector's mean occupations
+    const int owners = pass_warps(K) / L.ni;
+    const double fu = (double)h->nu / h->ns, fd = (double)h->nd / h->ns;
+    double total = 0.0, above = (fu + fd) * h->ns, run = 0.0;
+    std::vector<double> w(h->M);
+    for (int p = 0; p < h->M; ++p) {
+        const double f = p < h->ns ? fu : fd;
+        above -= f;
+        total += w[p] = f * above;
+    }
+    int f = 1;
+    for (int p = 0; p < h->M && f < owners; ++p) {
+        run += w[p];
+        while (f < owners && run >= total * f / owners) a.bounds[f++] = p + 1;
+    }
+    while (f <= owners) a.bounds[f++] = h->M;
+}
+
+// pass with FP64 sums over the FP64, FP32 or (gradient only) BF16 store
+static int launch_pass(vmc_ctx* h, const void* s_pf, int store_bytes, int K, bool gather, const double* V, double* T,
+                       const int* stop, cudaStream_t st, int* nblk) {
+    vmc_ctx::PassPlan* L;
+    int rc = plan_pass(h, K, gather, &L);
+    if (rc) return rc;
+    const int64_t need = (h->n_s + pass_warps(K) - 1) / pass_warps(K);
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(h->nsm, need));
+    if ((size_t)grid * h->npf * K * sizeof(double) > h->pfpart_bytes) return VMC_ERR_UNSUPPORTED;
+    vmc_ctx::PassRec rec{};
+    if (h->prof) {
+        rec.a = h->get_event();
+        rec.b = h->get_event();
+        rec.kind = store_bytes == 8 ? VMC_STORE_FP64 : store_bytes == 4 ? VMC_STORE_FP32 : VMC_STORE_BF16;
+        rec.bytes = (double)h->n_s * (2.0 * h->ncorr + h->N + (double)h->P * store_bytes);
+        VCK(cudaEventRecord(rec.a, st));
+    }
+    PassArgs a;
+    pass_args(h, *L, K, s_pf, V, T, stop, a);
+    VCK(launch_sr_pass(store_bytes, a, K, gather, grid, L->smem, st));
+    h->n_launch++;
+    if (h->prof) {
+        VCK(cudaEventRecord(rec.b, st));
+        h->recs.push_back(rec);
+    }
+    *nblk = grid;
+    return VMC_OK;
+}
+
+// generic pass with FP32 sums
+template <typename ST, int K>
+static int launch_main(vmc_ctx* h, const void* s_pf, const float* V, const float* invC, float* T, const int* stop,
                        cudaStream_t st, int* nblk) {
     const int threads = 512;
-    size_t smem = (size_t)h->npf * K * sizeof(AT) * (G ? 2 : 1) + (size_t)h->M * 4 + 16 * 64;
+    size_t smem = (size_t)h->npf * K * sizeof(float) * 2 + (size_t)h->M * 4 + 16 * 64;
     if (smem > h->smem_optin) { set_err("pairing block does not fit in shared memory"); return VMC_ERR_UNSUPPORTED; }
-    auto kern = k_sr_main<ST, AT, K, G>;
+    auto kern = k_sr_main<ST, K>;
     VCK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
     VCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
@@ -1181,10 +1272,8 @@ static int launch_main(vmc_ctx* h, const void* s_pf, const AT* V, const AT* invC
     int grid = h->nsm * per_sm;
     int64_t need = (h->n_s + 15) / 16;
     if (need < grid) grid = (int)std::max<int64_t>(1, need);
-    if ((size_t)grid * h->npf * K * sizeof(AT) > h->pfpart_bytes) return VMC_ERR_UNSUPPORTED;
-    const int kind = sizeof(ST) == 8 ? VMC_STORE_FP64
-                     : sizeof(ST) == 2 ? VMC_STORE_BF16
-                     : (sizeof(AT) == 8 ? VMC_STORE_FP32 : VMC_STORE_FP32_F32ACC);
+    if ((size_t)grid * h->npf * K * sizeof(float) > h->pfpart_bytes) return VMC_ERR_UNSUPPORTED;
+    const int kind = sizeof(ST) == 2 ? VMC_STORE_BF16 : VMC_STORE_FP32_F32ACC;
     vmc_ctx::PassRec rec{};
     if (h->prof) {
         rec.a = h->get_event();
@@ -1193,14 +1282,14 @@ static int launch_main(vmc_ctx* h, const void* s_pf, const AT* V, const AT* invC
         rec.bytes = (double)h->n_s * (2.0 * h->ncorr + h->N + (double)h->P * sizeof(ST));
         VCK(cudaEventRecord(rec.a, st));
     }
-    MainArgs<AT> a{};
+    MainArgs<float> a{};
     a.pb = h->pb;
     a.n_s = h->n_s;
     a.s_occ = h->d_socc; a.Nst = h->Nst;
     a.s_cidx = h->d_cidx; a.ncst = h->ncst;
     a.s_pf = s_pf; a.Pst = h->Pst;
     a.V = V; a.invC = invC; a.T = T;
-    a.pf_partial = (AT*)h->d_pfpart;
+    a.pf_partial = (float*)h->d_pfpart;
     a.stop = stop;
     kern<<<grid, threads, smem, st>>>(a);
     VCK(cudaGetLastError());
@@ -1725,7 +1814,10 @@ static int apply_S_impl(vmc_ctx* h, const void* s_pf, int kind, const AT* V, AT*
         if (rc == VMC_ERR_UNSUPPORTED && path != VMC_PATH_GENERIC && h->use_stream)
             rc = launch_stream<ST, K>(h, s_pf, (const float*)V, (const float*)invC, (float*)T, stop, st, &nblk);
     }
-    if (rc == VMC_ERR_UNSUPPORTED) rc = launch_main<ST, AT, K, true>(h, s_pf, V, invC, T, stop, st, &nblk);
+    if (rc == VMC_ERR_UNSUPPORTED) {
+        if constexpr (sizeof(AT) == 8) rc = launch_pass(h, s_pf, (int)sizeof(ST), K, true, V, T, stop, st, &nblk);
+        else rc = launch_main<ST, K>(h, s_pf, V, invC, T, stop, st, &nblk);
+    }
     if (rc) return rc;
     if (!sorted) {   // the sorted pass scatters the correlators itself
         rc = launch_corr<AT, K>(h, T, stop, st);
@@ -1778,9 +1870,7 @@ static int gradient_pass(vmc_ctx* h, int kind, double* g, cudaStream_t st) {
     k_build_T_grad<<<kNumPart, 256, 0, st>>>(h->d_E, h->n_s, T, h->part(1)); h->n_launch++;
     VCK(cudaGetLastError());
     int nblk = 0, rc;
-    if (kind == 0) rc = launch_main<double, double, 2, false>(h, src, nullptr, nullptr, T, nullptr, st, &nblk);
-    else if (kind == 1) rc = launch_main<float, double, 2, false>(h, src, nullptr, nullptr, T, nullptr, st, &nblk);
-    else rc = launch_main<__nv_bfloat16, double, 2, false>(h, src, nullptr, nullptr, T, nullptr, st, &nblk);
+    rc = launch_pass(h, src, kind == 0 ? 8 : kind == 1 ? 4 : 2, 2, false, nullptr, T, nullptr, st, &nblk);
     if (rc) return rc;
     rc = launch_corr<double, 2>(h, T, nullptr, st);
     if (rc) return rc;
@@ -1855,6 +1945,7 @@ extern "C" int sr_gradient(vmc_handle h, double* g, double* e_stats, int store, 
 }
 
 static size_t main_smem(const vmc_ctx* h, int K, size_t at_bytes) {
+    if (at_bytes == 8) return pass_smem(h->npf, h->P, K, true, 1);
     return (size_t)h->npf * K * at_bytes * 2 + (size_t)h->M * 4 + 16 * 64;
 }
 
@@ -2910,7 +3001,7 @@ extern "C" int sr_apply_S_batch(const vmc_handle* hs, int n, const double* const
     }
     vmc_ctx* h0 = hs[0];
     cudaStream_t st = (cudaStream_t)stream;
-    std::vector<MainArgs<double>> args(n);
+    std::vector<PassArgs> args(n);
     std::vector<int> cta0(n + 1, 0);
     // CTAs in proportion to each problem's stored bytes, about two per SM in all
     size_t smem = 0;
@@ -2922,32 +3013,25 @@ extern "C" int sr_apply_S_batch(const vmc_handle* hs, int n, const double* const
         if (rc) return rc;
         k_dot_part<double, double, 1><<<vgrid(h, 1), 256, 0, st>>>(h->d_Obar[kind], V[b], h->nv, h->part(0), nullptr);
         h->n_launch++;
-        smem = std::max(smem, main_smem(h, 1, sizeof(double)));
+        vmc_ctx::PassPlan* L;
+        if ((rc = plan_pass(h, 1, true, &L))) return rc;
+        smem = std::max(smem, L->smem);
         const double share = (double)h->n_s * (h->P + h->ncorr) / work;
         int g = (int)std::ceil(share * 2 * h0->nsm);
         g = (int)std::max<int64_t>(1, std::min<int64_t>(g, (h->n_s + 15) / 16));
         g = std::min<int64_t>(g, (int64_t)(h->pfpart_bytes / ((size_t)h->npf * sizeof(double))));
         cta0[b + 1] = cta0[b] + g;
-        MainArgs<double>& a = args[b];
-        a.pb = h->pb;
-        a.n_s = h->n_s;
-        a.s_occ = h->d_socc; a.Nst = h->Nst;
-        a.s_cidx = h->d_cidx; a.ncst = h->ncst;
-        a.s_pf = store_ptr(h, kind); a.Pst = h->Pst;
-        a.V = V[b]; a.invC = h->d_invC64; a.T = (double*)h->d_T;
-        a.pf_partial = (double*)h->d_pfpart;
-        a.stop = nullptr;
+        pass_args(h, *L, 1, store_ptr(h, kind), V[b], (double*)h->d_T, nullptr, args[b]);
     }
-    if (smem > h0->smem_optin) { set_err("pairing block does not fit in shared memory"); return VMC_ERR_UNSUPPORTED; }
     void* dbuf = nullptr;
-    const size_t abytes = round_up(sizeof(MainArgs<double>) * n, 256);
+    const size_t abytes = round_up(sizeof(PassArgs) * n, 256);
     int rc = batch_buffer(h0, abytes + sizeof(int) * (n + 1), &dbuf);
     if (rc) return rc;
-    MainArgs<double>* dargs = (MainArgs<double>*)dbuf;
+    PassArgs* dargs = (PassArgs*)dbuf;
     int* dcta = (int*)((unsigned char*)dbuf + abytes);
-    VCK(cudaMemcpyAsync(dargs, args.data(), sizeof(MainArgs<double>) * n, cudaMemcpyHostToDevice, st));
+    VCK(cudaMemcpyAsync(dargs, args.data(), sizeof(PassArgs) * n, cudaMemcpyHostToDevice, st));
     VCK(cudaMemcpyAsync(dcta, cta0.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, st));
-    VCK(launch_sr_main_batch(kind == 0 ? 8 : 4, cta0[n], smem, st, dargs, dcta, n));
+    VCK(launch_sr_pass_batch(kind == 0 ? 8 : 4, cta0[n], smem, st, dargs, dcta, n));
     h0->n_launch++;
     for (int b = 0; b < n; ++b) {
         vmc_ctx* h = hs[b];

@@ -111,10 +111,10 @@ __global__ void k_logpsi(LogPsiArgs a);
 // ---------------------------------------------------------------------------
 enum StoreKind { STORE_F64 = 0, STORE_F32 = 1, STORE_BF16 = 2 };
 
-// Streaming pass over the O store.  With GATHER, t_s = O_s . V for K vectors
-// (correlator gather + pairing-block dot) is computed and written to T;
-// otherwise t_s is read from T.  Then sum_s t_s O_s restricted to the
-// pairing block is accumulated per CTA and written to pf_partial[cta].
+// Streaming pass over the O store: t_s = O_s . V for K vectors (correlator
+// gather + pairing-block dot) is computed and written to T, then sum_s t_s O_s
+// restricted to the pairing block is accumulated per CTA and written to
+// pf_partial[cta].
 template <typename AT>
 struct MainArgs {
     DevProblem pb;
@@ -131,6 +131,33 @@ struct MainArgs {
     AT* pf_partial;       // [gridDim][npf][K]
     const int* stop;      // early exit flag (may be null)
 };
+
+// The same with FP64 sums and no atomics (pass.cu), or for the gradient K = 2
+// with t_s read from T.
+constexpr int pass_warps(int K) { return K == 4 ? 16 : 32; }   // warps per CTA (one CTA per SM)
+constexpr int kPassTile = 32;    // samples between barriers
+struct PassArgs {
+    DevProblem pb;
+    int64_t n_s;
+    const uint8_t* s_occ;
+    int Nst;
+    const cstate_t* s_cidx;
+    int ncst;
+    const void* s_pf;
+    int64_t Pst;
+    const uint32_t* fulltab;  // [P] element e | a << 16 | b << 24 in row-major order of the pairs a < b
+    const double* V;          // [K][nv]
+    const double* invC;       // [ncp]
+    double* T;                // [n_s][K]
+    double* pf_partial;       // [gridDim][npf][K]
+    int ni;                   // images; pass_warps(K) / ni warps share one
+    int bounds[pass_warps(1) + 1];   // first orbital p of each of an image's owners, then M
+    const int* stop;
+};
+size_t pass_smem(int npf, int P, int K, bool gather, int ni);
+cudaError_t launch_sr_pass(int store_bytes, const PassArgs& a, int K, bool gather, int grid, size_t smem, cudaStream_t st);
+cudaError_t launch_sr_pass_batch(int store_bytes, int blocks, size_t smem, cudaStream_t st, const PassArgs* args,
+                                 const int* cta0, int n);
 
 template <typename AT>
 struct CorrArgs {
@@ -171,10 +198,7 @@ struct FinArgs {
 };
 
 
-template <typename ST, typename AT, int K, bool GATHER>
-__global__ void __launch_bounds__(512) k_sr_main(MainArgs<AT> a);
-cudaError_t launch_sr_main_batch(int store_bytes, int blocks, size_t smem, cudaStream_t st,
-                                 const MainArgs<double>* args, const int* cta0, int n);
+template <typename ST, int K> __global__ void __launch_bounds__(512) k_sr_main(MainArgs<float> a);
 template <typename AT, int K>
 __global__ void __cluster_dims__(kCorrCluster, 1, 1) __launch_bounds__(256) k_corr_scatter(CorrArgs<AT> a);
 template <typename AT, int K> __global__ void __launch_bounds__(256) k_corr_scatter_global(CorrArgs<AT> a);

@@ -1,0 +1,289 @@
+// One-pass Eq. 7 product and gradient pass over the O store with FP64 sums
+// (FP64 arithmetic; FP32 pairs for the FP32 store), without atomics.
+//
+// A CTA works through its samples in tiles.  Gather: a warp per sample forms
+// t_s = O_s . V.  Scatter: t_s O_s is added to shared-memory images of the
+// pairing block.  An image belongs to `owners` warps that split the samples'
+// elements by their smaller orbital p = occ[a] (boundaries of about equal
+// expected work), so two warps never touch one address, whatever samples they
+// are at: an update is a plain load, add and store, and the only
+// synchronisation is one barrier per tile between gather and scatter.  There
+// are as many images as shared memory holds (two at 128 spin orbitals, one
+// per warp on small lattices, where a warp keeps its sample for both halves
+// and needs no barrier).  The sums have a fixed order.
+//
+// What bounds it: the FP64 store's pass the FP64 pipe (two FMAs per element, 72 %
+// busy), the FP32 store's issue slots and shared-memory latency (32 warps).  8x8
+// lattice, 28 + 28 electrons: FP64 store, 65,536 samples 600 us (825 us with FP64
+// shared atomics), FP32 store, 131,072 samples 930 us (1,299 us with two shared
+// FP32 atomics per element).  Warps per CTA: 16 695 / 1,225 us, 32 600 / 930 us;
+// the FP32 store's gather in FP64 1,470 us (conversions fill the FP64 pipe);
+// scatter rounds of 4 elements per lane, skipped by the whole warp, 643 / 976 us.
+//
+// Elements go in the row-major order of electron pairs a < b (fulltab), in
+// which an owner's share of a sample is one stretch; the tile's occupations
+// and row bases sit in shared memory.  The second read of the values comes out
+// of L2.
+//
+// FP32 pairs: the FP64 pipe of this GPU retires one warp FMA per 16 cycles per
+// SM, so the FP32 store's passes stay off it.  The v table holds
+// each FP64 value as an FP32 pair (hi, lo); a product w v = w hi + w lo is
+// split exactly into its rounded value and the FMA error term; the per-lane
+// sums and the images are FP32 pairs kept by Knuth's two-sum.  The rounded
+// intrinsics keep the compiler from fusing the error arithmetic.
+#include <type_traits>
+#include "common.cuh"
+#include "kernels.h"
+
+namespace vmc {
+
+namespace {
+
+__device__ __forceinline__ void ff_add(float& sh, float& sl, float p, float err) {
+    const float s = __fadd_rn(sh, p);
+    const float bp = __fsub_rn(s, sh);
+    const float e = __fadd_rn(__fsub_rn(sh, __fsub_rn(s, bp)), __fsub_rn(p, bp));
+    sh = s;
+    sl = __fadd_rn(sl, __fadd_rn(e, err));
+}
+
+__device__ __forceinline__ float2 ff_split(double v) {
+    const float h = (float)v;
+    return make_float2(h, (float)(v - (double)h));
+}
+
+__device__ __forceinline__ float load_w(const float* p) { return __ldg(p); }
+__device__ __forceinline__ double load_w(const double* p) { return __ldg(p); }
+__device__ __forceinline__ float load_w(const __nv_bfloat16* p) {
+    return __uint_as_float((uint32_t)__ldg((const unsigned short*)p) << 16);
+}
+// FP32 to FP64 by its bits (a conversion would take the FP64 pipe's time again)
+__device__ __forceinline__ double widen(double w) { return w; }
+__device__ __forceinline__ double widen(float w) {
+    const uint32_t u = __float_as_uint(w), m = u & 0x7fffffffu;
+    double d = __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+    if (__any_sync(__activemask(), m - 0x00800000u >= 0x7f000000u)) d = (double)w;   // not a normal number in some lane
+    return d;
+}
+
+// Element arithmetic: plain FP64, or FP32 pairs for the FP32 store.
+struct PlainAcc {
+    using Elem = double;   // a table or image entry
+    static __device__ __forceinline__ Elem make(double v) { return v; }
+    static __device__ __forceinline__ double value(Elem v) { return v; }
+    template <typename W> static __device__ __forceinline__ void add(Elem& s, W w, Elem v) { s = fma(widen(w), v, s); }
+};
+struct PairAcc {
+    using Elem = float2;
+    static __device__ __forceinline__ Elem make(double v) { return ff_split(v); }
+    static __device__ __forceinline__ double value(Elem v) { return (double)v.x + (double)v.y; }
+    static __device__ __forceinline__ void add(Elem& s, float w, Elem v) {
+        const float p = __fmul_rn(w, v.x);
+        ff_add(s.x, s.y, p, fmaf(w, v.y, fmaf(w, v.x, -p)));
+    }
+};
+
+constexpr int kU = 4, kUs = 2;   // elements per lane in flight, gather and scatter
+
+// shared memory of one tile buffer
+template <typename E, int K, int NW>
+struct TileBuf {
+    E t[kPassTile][K];
+    int16_t rb[kPassTile][64];               // row bases of the occupied orbitals
+    uint8_t occ[kPassTile][64];
+    uint16_t start[kPassTile][NW + 1];   // first element (rank) of each owner
+};
+
+template <typename ST, int K, bool GATHER, int NW>
+__device__ void pass_run(const PassArgs& a, int cta, int ncta, unsigned char* smem) {
+    using A = typename std::conditional<std::is_same<ST, float>::value, PairAcc, PlainAcc>::type;
+    using E = typename A::Elem;
+    const DevProblem& pb = a.pb;
+    const int npf = pb.npf, N = pb.N, P = pb.P, ni = a.ni, owners = NW / ni;
+    E* img = (E*)smem;                                           // [ni][npf][K]
+    E* vpf = img + (size_t)ni * npf * K;                         // [npf][K]
+    TileBuf<E, K, NW>* buf = (TileBuf<E, K, NW>*)(vpf + (GATHER ? (size_t)npf * K : 0));   // [2]
+    uint32_t* ft = (uint32_t*)(buf + 2);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < ni * npf * K; i += blockDim.x) img[i] = A::make(0.0);
+    if (GATHER)
+        for (int i = threadIdx.x; i < npf; i += blockDim.x)
+#pragma unroll
+            for (int kk = 0; kk < K; ++kk) vpf[i * K + kk] = A::make(a.V[kk * pb.nv + pb.ncp + i]);
+    for (int i = threadIdx.x; i < P; i += blockDim.x) ft[i] = a.fulltab[i];
+    __syncthreads();
+    const ST* pf = (const ST*)a.s_pf;
+    const int im = wid / owners, own = wid % owners;
+    E* my = img + (size_t)im * npf * K;
+    const int64_t per = (a.n_s + ncta - 1) / ncta;
+    const int64_t s0 = min(a.n_s, cta * per), s1 = min(a.n_s, s0 + per);
+    int cur = 0;
+    for (int64_t sb = s0; sb < s1; sb += kPassTile, cur ^= 1) {
+        TileBuf<E, K, NW>& B = buf[cur];
+        const int n = (int)min((int64_t)kPassTile, s1 - sb);
+        // ---- gather: the warp's samples of the tile ------------------------
+        for (int j = wid; j < n; j += NW) {
+            const int64_t s = sb + j;
+            int o[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int i = lane + 32 * h;
+                o[h] = i < N ? a.s_occ[s * a.Nst + i] : 255;
+                if (i < N) {
+                    B.occ[j][i] = (uint8_t)o[h];
+                    B.rb[j][i] = (int16_t)pf_row_base(pb.M, o[h]);
+                }
+            }
+            for (int f = 0; f <= owners; ++f) {   // a = electrons below the owner's first orbital
+                const int a0 = __popc(__ballot_sync(VMC_FULL_MASK, o[0] < a.bounds[f])) +
+                               __popc(__ballot_sync(VMC_FULL_MASK, o[1] < a.bounds[f]));
+                if (lane == 0) B.start[j][f] = (uint16_t)(a0 * (2 * N - a0 - 1) / 2);
+            }
+            __syncwarp();
+            if (GATHER) {
+                E sum[K];
+                double tc[K];
+#pragma unroll
+                for (int kk = 0; kk < K; ++kk) {
+                    sum[kk] = A::make(0.0);
+                    tc[kk] = 0.0;
+                }
+                for (int c = lane; c < pb.ncorr; c += 32) {
+                    const int64_t k = pb.corr_off[c] + a.s_cidx[s * a.ncst + c];
+                    const double ic = a.invC[k];
+#pragma unroll
+                    for (int kk = 0; kk < K; ++kk) tc[kk] += a.V[kk * pb.nv + k] * ic;
+                }
+                const ST* row = pf + s * a.Pst;
+                for (int r0 = lane; r0 < P; r0 += 32 * kU) {
+                    decltype(load_w(row)) w[kU];
+                    int pq[kU];
+#pragma unroll
+                    for (int u = 0; u < kU; ++u) {
+                        const uint32_t f = ft[min(r0 + 32 * u, P - 1)];
+                        w[u] = load_w(row + (f & 0xFFFFu));
+                        pq[u] = B.rb[j][(f >> 16) & 255] + B.occ[j][f >> 24];
+                    }
+#pragma unroll
+                    for (int u = 0; u < kU; ++u)
+                        if (r0 + 32 * u < P)
+#pragma unroll
+                            for (int kk = 0; kk < K; ++kk) A::add(sum[kk], w[u], vpf[pq[u] * K + kk]);
+                }
+#pragma unroll
+                for (int kk = 0; kk < K; ++kk) {
+                    const double t = warp_sum(A::value(sum[kk]) + tc[kk]);
+                    if (lane == 0) {
+                        a.T[s * K + kk] = t;
+                        B.t[j][kk] = A::make(t);
+                    }
+                }
+            } else if (lane < K) {
+                B.t[j][lane] = A::make(a.T[s * K + lane]);
+            }
+        }
+        if (owners > 1) __syncthreads();
+        else __syncwarp();
+        // ---- scatter: the owner's share of the image's samples ---------------
+        for (int j = im; j < n; j += ni) {
+            const ST* row = pf + (sb + j) * a.Pst;
+            E t[K];
+#pragma unroll
+            for (int kk = 0; kk < K; ++kk) t[kk] = B.t[j][kk];
+            const int r1 = B.start[j][own + 1];
+            for (int r0 = B.start[j][own] + lane; r0 < r1; r0 += 32 * kUs) {
+                decltype(load_w(row)) w[kUs];
+                int pq[kUs];
+#pragma unroll
+                for (int u = 0; u < kUs; ++u) {
+                    const uint32_t f = ft[min(r0 + 32 * u, P - 1)];
+                    w[u] = load_w(row + (f & 0xFFFFu));
+                    pq[u] = B.rb[j][(f >> 16) & 255] + B.occ[j][f >> 24];
+                }
+                E x[kUs][K];   // a sample's elements are at distinct addresses: loads first
+#pragma unroll
+                for (int u = 0; u < kUs; ++u)
+#pragma unroll
+                    for (int kk = 0; kk < K; ++kk) x[u][kk] = my[pq[u] * K + kk];
+#pragma unroll
+                for (int u = 0; u < kUs; ++u)
+                    if (r0 + 32 * u < r1)
+#pragma unroll
+                        for (int kk = 0; kk < K; ++kk) {
+                            A::add(x[u][kk], w[u], t[kk]);
+                            my[pq[u] * K + kk] = x[u][kk];
+                        }
+            }
+            __syncwarp();   // the next sample's elements may meet these addresses in other lanes
+        }
+    }
+    __syncthreads();
+    double* dst = a.pf_partial + (size_t)cta * npf * K;
+    for (int i = threadIdx.x; i < npf * K; i += blockDim.x) {
+        double x = 0.0;
+        for (int k = 0; k < ni; ++k) x += A::value(img[(size_t)k * npf * K + i]);
+        dst[i] = x;
+    }
+}
+
+template <typename ST, int K, bool GATHER>
+__global__ void __launch_bounds__(32 * pass_warps(K), 1) k_sr_pass(PassArgs a) {
+    if (a.stop && *a.stop) return;
+    extern __shared__ __align__(16) unsigned char smem[];
+    pass_run<ST, K, GATHER, pass_warps(K)>(a, blockIdx.x, gridDim.x, smem);
+}
+
+// Several problems in one launch: CTAs [cta0[b], cta0[b + 1]) serve problem
+// b, each with the shared-memory layout of its own problem.
+template <typename ST>
+__global__ void __launch_bounds__(32 * pass_warps(1), 1) k_sr_pass_batch(const PassArgs* __restrict__ args,
+                                                                         const int* __restrict__ cta0, int n) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    int b = 0;
+    while (b + 1 < n && (int)blockIdx.x >= cta0[b + 1]) ++b;
+    if ((int)blockIdx.x >= cta0[n]) return;
+    pass_run<ST, 1, true, pass_warps(1)>(args[b], blockIdx.x - cta0[b], cta0[b + 1] - cta0[b], smem);
+}
+
+template <typename ST, int K, bool GATHER>
+cudaError_t launch(const PassArgs& a, int grid, size_t smem, cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(k_sr_pass<ST, K, GATHER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_sr_pass<ST, K, GATHER><<<grid, 32 * pass_warps(K), smem, st>>>(a);
+    return cudaGetLastError();
+}
+
+template <typename ST>
+cudaError_t launch_k(const PassArgs& a, int K, bool gather, int grid, size_t smem, cudaStream_t st) {
+    if (!gather) return launch<ST, 2, false>(a, grid, smem, st);
+    if (K == 1) return launch<ST, 1, true>(a, grid, smem, st);
+    if (K == 2) return launch<ST, 2, true>(a, grid, smem, st);
+    return launch<ST, 4, true>(a, grid, smem, st);
+}
+
+}  // namespace
+
+// shared memory with ni images (a table or image entry is 8 bytes in either arithmetic)
+size_t pass_smem(int npf, int P, int K, bool gather, int ni) {
+    const size_t tile = K == 1   ? sizeof(TileBuf<double, 1, pass_warps(1)>)
+                        : K == 2 ? sizeof(TileBuf<double, 2, pass_warps(2)>)
+                                 : sizeof(TileBuf<double, 4, pass_warps(4)>);
+    return (size_t)npf * K * 8 * (ni + (gather ? 1 : 0)) + 2 * tile + (size_t)P * 4;
+}
+
+cudaError_t launch_sr_pass(int store_bytes, const PassArgs& a, int K, bool gather, int grid, size_t smem, cudaStream_t st) {
+    if (store_bytes == 8) return launch_k<double>(a, K, gather, grid, smem, st);
+    if (store_bytes == 4) return launch_k<float>(a, K, gather, grid, smem, st);
+    return launch<__nv_bfloat16, 2, false>(a, grid, smem, st);   // the BF16 store's means only
+}
+
+cudaError_t launch_sr_pass_batch(int store_bytes, int blocks, size_t smem, cudaStream_t st, const PassArgs* args,
+                                 const int* cta0, int n) {
+    auto kern = store_bytes == 8 ? k_sr_pass_batch<double> : k_sr_pass_batch<float>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<blocks, 32 * pass_warps(1), smem, st>>>(args, cta0, n);
+    return cudaGetLastError();
+}
+
+}  // namespace vmc

@@ -22,241 +22,73 @@
 
 namespace vmc {
 
-template <typename ST, typename AT> __device__ __forceinline__ AT load_st(const void* p, int64_t i);
-template <> __device__ __forceinline__ double load_st<double, double>(const void* p, int64_t i) {
-    return __ldg((const double*)p + i);
-}
-template <> __device__ __forceinline__ double load_st<float, double>(const void* p, int64_t i) {
-    return (double)__ldg((const float*)p + i);
-}
-template <> __device__ __forceinline__ float load_st<float, float>(const void* p, int64_t i) {
+template <typename ST> __device__ __forceinline__ float load_st(const void* p, int64_t i);
+template <> __device__ __forceinline__ float load_st<float>(const void* p, int64_t i) {
     return __ldg((const float*)p + i);
 }
-template <> __device__ __forceinline__ float load_st<__nv_bfloat16, float>(const void* p, int64_t i) {
+template <> __device__ __forceinline__ float load_st<__nv_bfloat16>(const void* p, int64_t i) {
     return __bfloat162float(((const __nv_bfloat16*)p)[i]);
 }
-template <> __device__ __forceinline__ double load_st<__nv_bfloat16, double>(const void* p, int64_t i) {
-    return (double)__bfloat162float(((const __nv_bfloat16*)p)[i]);
-}
 
-// FP32 store with FP64-accurate sums in FP32 arithmetic.  The FP64 pipe of
-// this GPU retires one warp FMA per 16 cycles per SM, and the FP64 form of
-// this pass (conversions, FMAs and FP64 shared atomics) is bound by it.
-// Here the v table holds each FP64 value as an FP32 pair (hi, lo); a product
-// w v = w hi + w lo is split exactly into its rounded value and the FMA error
-// term; the per-lane sums are FP32 pairs kept by Knuth's two-sum; the image
-// of the pairing block is two FP32 arrays: the first atomic add returns the
-// old value, so the rounding error of the add it made is known exactly and
-// is added to the second array with the product's error terms.  The rounded
-// intrinsics keep the compiler from fusing the error arithmetic.
-__device__ __forceinline__ void ff_add(float& sh, float& sl, float p, float err) {
-    const float s = __fadd_rn(sh, p);
-    const float bp = __fsub_rn(s, sh);
-    const float e = __fadd_rn(__fsub_rn(sh, __fsub_rn(s, bp)), __fsub_rn(p, bp));
-    sh = s;
-    sl = __fadd_rn(sl, __fadd_rn(e, err));
-}
-
-template <int K, bool GATHER>
-__device__ void sr_main_run_ff(const MainArgs<double>& a, int cta, int ncta, unsigned char* smem) {
+// The generic pass with FP32 sums: a warp per sample, shared atomics into an
+// image per CTA.  (Passes with FP64 sums: pass.cu.)
+template <typename ST, int K>
+__global__ void __launch_bounds__(512) k_sr_main(MainArgs<float> a) {
+    if (a.stop && *a.stop) return;
+    extern __shared__ __align__(16) unsigned char smem[];
     const DevProblem& pb = a.pb;
     const int npf = pb.npf, M = pb.M, N = pb.N, P = pb.P;
-    float* hi = (float*)smem;                    // [npf][K] image, rounded sums
-    float* lo = hi + (size_t)npf * K;            // [npf][K] their rounding errors
-    float2* vpf = (float2*)(lo + (size_t)npf * K);
-    int* rowbase = (int*)(vpf + (GATHER ? (size_t)npf * K : 0));
+    float* acc = (float*)smem;
+    float* vpf = acc + (size_t)npf * K;
+    int* rowbase = (int*)(vpf + (size_t)npf * K);
     uint8_t* occw = (uint8_t*)(rowbase + M);
-    for (int i = threadIdx.x; i < 2 * npf * K; i += blockDim.x) hi[i] = 0.f;
-    if (GATHER)
-        for (int i = threadIdx.x; i < npf; i += blockDim.x)
+    for (int i = threadIdx.x; i < npf * K; i += blockDim.x) acc[i] = 0.f;
+    for (int i = threadIdx.x; i < npf; i += blockDim.x)
 #pragma unroll
-            for (int kk = 0; kk < K; ++kk) {
-                const double v = a.V[kk * pb.nv + pb.ncp + i];
-                const float vh = (float)v;
-                vpf[i * K + kk] = make_float2(vh, (float)(v - (double)vh));
-            }
+        for (int kk = 0; kk < K; ++kk) vpf[i * K + kk] = a.V[kk * pb.nv + pb.ncp + i];
     for (int i = threadIdx.x; i < M; i += blockDim.x) rowbase[i] = pb.rowbase[i];
     __syncthreads();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     uint8_t* my = occw + wid * 64;
-    const float* pf = (const float*)a.s_pf;
-    for (int64_t s = (int64_t)cta * nw + wid; s < a.n_s; s += (int64_t)ncta * nw) {
+    for (int64_t s = (int64_t)blockIdx.x * nw + wid; s < a.n_s; s += (int64_t)gridDim.x * nw) {
         for (int i = lane; i < N; i += 32) my[i] = a.s_occ[s * a.Nst + i];
         __syncwarp();
-        double t[K];
-        if (GATHER) {
-            double tc[K];
-            float sh[K], sl[K];
+        float t[K];
 #pragma unroll
-            for (int kk = 0; kk < K; ++kk) {
-                tc[kk] = 0.0;
-                sh[kk] = sl[kk] = 0.f;
-            }
-            for (int c = lane; c < pb.ncorr; c += 32) {
-                const int64_t k = pb.corr_off[c] + a.s_cidx[s * a.ncst + c];
-                const double ic = a.invC[k];
+        for (int kk = 0; kk < K; ++kk) t[kk] = 0.f;
+        for (int c = lane; c < pb.ncorr; c += 32) {
+            int64_t k = pb.corr_off[c] + a.s_cidx[s * a.ncst + c];
+            float ic = a.invC[k];
 #pragma unroll
-                for (int kk = 0; kk < K; ++kk) tc[kk] += a.V[kk * pb.nv + k] * ic;
-            }
-            // four elements per lane in flight: the loads first
-            for (int e0 = lane; e0 < P; e0 += 128) {
-                int pq[4];
-                float w[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int e = e0 + 32 * u;
-                    w[u] = e < P ? __ldg(pf + s * a.Pst + e) : 0.f;
-                    const uint16_t pt = e < P ? pb.pairtab[e] : (uint16_t)0;
-                    pq[u] = rowbase[my[pt & 255]] + my[pt >> 8];
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    if (e0 + 32 * u >= P) continue;
-#pragma unroll
-                    for (int kk = 0; kk < K; ++kk) {
-                        const float2 v = vpf[pq[u] * K + kk];
-                        const float p = __fmul_rn(w[u], v.x);
-                        ff_add(sh[kk], sl[kk], p, __fadd_rn(fmaf(w[u], v.x, -p), __fmul_rn(w[u], v.y)));
-                    }
-                }
-            }
-#pragma unroll
-            for (int kk = 0; kk < K; ++kk) t[kk] = warp_sum((double)sh[kk] + (double)sl[kk] + tc[kk]);
-            if (lane < K) {
-                double mine = t[0];
-#pragma unroll
-                for (int kk = 1; kk < K; ++kk) if (lane == kk) mine = t[kk];
-                a.T[s * K + lane] = mine;
-            }
-        } else {
-#pragma unroll
-            for (int kk = 0; kk < K; ++kk) t[kk] = a.T[s * K + kk];
-        }
-        float th[K], tl[K];
-#pragma unroll
-        for (int kk = 0; kk < K; ++kk) {
-            th[kk] = (float)t[kk];
-            tl[kk] = (float)(t[kk] - (double)th[kk]);
-        }
-        for (int e0 = lane; e0 < P; e0 += 128) {
-            int pq[4];
-            float w[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int e = e0 + 32 * u;
-                w[u] = e < P ? __ldg(pf + s * a.Pst + e) : 0.f;
-                const uint16_t pt = e < P ? pb.pairtab[e] : (uint16_t)0;
-                pq[u] = rowbase[my[pt & 255]] + my[pt >> 8];
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (e0 + 32 * u >= P) continue;
-#pragma unroll
-                for (int kk = 0; kk < K; ++kk) {
-                    const float p = __fmul_rn(th[kk], w[u]);
-                    const float err = __fadd_rn(fmaf(th[kk], w[u], -p), __fmul_rn(tl[kk], w[u]));
-                    const float old = atomicAdd(&hi[pq[u] * K + kk], p);
-                    const float sum = __fadd_rn(old, p);
-                    const float bp = __fsub_rn(sum, old);
-                    const float e2 = __fadd_rn(__fsub_rn(old, __fsub_rn(sum, bp)), __fsub_rn(p, bp));
-                    atomicAdd(&lo[pq[u] * K + kk], __fadd_rn(e2, err));
-                }
-            }
-        }
-        __syncwarp();
-    }
-    __syncthreads();
-    double* dst = a.pf_partial + (size_t)cta * npf * K;
-    for (int i = threadIdx.x; i < npf * K; i += blockDim.x) dst[i] = (double)hi[i] + (double)lo[i];
-}
-
-// The generic pass for one problem, run by CTA `cta` of `ncta` serving it.
-template <typename ST, typename AT, int K, bool GATHER>
-__device__ void sr_main_run(const MainArgs<AT>& a, int cta, int ncta, unsigned char* smem) {
-    if constexpr (std::is_same<ST, float>::value && std::is_same<AT, double>::value) {
-        if (a.pb.ff_sums) {
-            sr_main_run_ff<K, GATHER>(a, cta, ncta, smem);
-            return;
-        }
-    }
-    const DevProblem& pb = a.pb;
-    const int npf = pb.npf, M = pb.M, N = pb.N, P = pb.P;
-    AT* acc = (AT*)smem;
-    AT* vpf = acc + (size_t)npf * K;
-    int* rowbase = (int*)(vpf + (GATHER ? (size_t)npf * K : 0));
-    uint8_t* occw = (uint8_t*)(rowbase + M);
-    for (int i = threadIdx.x; i < npf * K; i += blockDim.x) acc[i] = AT(0);
-    if (GATHER)
-        for (int i = threadIdx.x; i < npf; i += blockDim.x)
-#pragma unroll
-            for (int kk = 0; kk < K; ++kk) vpf[i * K + kk] = a.V[kk * pb.nv + pb.ncp + i];
-    for (int i = threadIdx.x; i < M; i += blockDim.x) rowbase[i] = pb.rowbase[i];
-    __syncthreads();
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    uint8_t* my = occw + wid * 64;
-    for (int64_t s = (int64_t)cta * nw + wid; s < a.n_s; s += (int64_t)ncta * nw) {
-        for (int i = lane; i < N; i += 32) my[i] = a.s_occ[s * a.Nst + i];
-        __syncwarp();
-        AT t[K];
-        if (GATHER) {
-#pragma unroll
-            for (int kk = 0; kk < K; ++kk) t[kk] = AT(0);
-            for (int c = lane; c < pb.ncorr; c += 32) {
-                int64_t k = pb.corr_off[c] + a.s_cidx[s * a.ncst + c];
-                AT ic = a.invC[k];
-#pragma unroll
-                for (int kk = 0; kk < K; ++kk) t[kk] += a.V[kk * pb.nv + k] * ic;
-            }
-            for (int e = lane; e < P; e += 32) {
-                uint16_t pt = pb.pairtab[e];
-                int pq = rowbase[my[pt & 255]] + my[pt >> 8];
-                AT w = load_st<ST, AT>(a.s_pf, s * a.Pst + e);
-#pragma unroll
-                for (int kk = 0; kk < K; ++kk) t[kk] += w * vpf[pq * K + kk];
-            }
-#pragma unroll
-            for (int kk = 0; kk < K; ++kk) t[kk] = warp_sum(t[kk]);
-            if (lane < K) {
-                AT mine = t[0];
-#pragma unroll
-                for (int kk = 1; kk < K; ++kk) if (lane == kk) mine = t[kk];
-                a.T[s * K + lane] = mine;
-            }
-        } else {
-#pragma unroll
-            for (int kk = 0; kk < K; ++kk) t[kk] = a.T[s * K + kk];
+            for (int kk = 0; kk < K; ++kk) t[kk] += a.V[kk * pb.nv + k] * ic;
         }
         for (int e = lane; e < P; e += 32) {
             uint16_t pt = pb.pairtab[e];
             int pq = rowbase[my[pt & 255]] + my[pt >> 8];
-            AT w = load_st<ST, AT>(a.s_pf, s * a.Pst + e);
+            float w = load_st<ST>(a.s_pf, s * a.Pst + e);
+#pragma unroll
+            for (int kk = 0; kk < K; ++kk) t[kk] += w * vpf[pq * K + kk];
+        }
+#pragma unroll
+        for (int kk = 0; kk < K; ++kk) t[kk] = warp_sum(t[kk]);
+        if (lane < K) {
+            float mine = t[0];
+#pragma unroll
+            for (int kk = 1; kk < K; ++kk) if (lane == kk) mine = t[kk];
+            a.T[s * K + lane] = mine;
+        }
+        for (int e = lane; e < P; e += 32) {
+            uint16_t pt = pb.pairtab[e];
+            int pq = rowbase[my[pt & 255]] + my[pt >> 8];
+            float w = load_st<ST>(a.s_pf, s * a.Pst + e);
 #pragma unroll
             for (int kk = 0; kk < K; ++kk) atomicAdd(&acc[pq * K + kk], t[kk] * w);
         }
         __syncwarp();
     }
     __syncthreads();
-    AT* dst = a.pf_partial + (size_t)cta * npf * K;
+    float* dst = a.pf_partial + (size_t)blockIdx.x * npf * K;
     for (int i = threadIdx.x; i < npf * K; i += blockDim.x) dst[i] = acc[i];
-}
-
-template <typename ST, typename AT, int K, bool GATHER>
-__global__ void __launch_bounds__(512) k_sr_main(MainArgs<AT> a) {
-    if (a.stop && *a.stop) return;
-    extern __shared__ __align__(16) unsigned char smem[];
-    sr_main_run<ST, AT, K, GATHER>(a, blockIdx.x, gridDim.x, smem);
-}
-
-// Several problems in one launch: CTAs [cta0[b], cta0[b + 1]) serve problem
-// b, each with the shared-memory layout of its own problem.
-template <typename ST, typename AT>
-__global__ void __launch_bounds__(512) k_sr_main_batch(const MainArgs<AT>* __restrict__ args,
-                                                       const int* __restrict__ cta0, int n) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    int b = 0;
-    while (b + 1 < n && (int)blockIdx.x >= cta0[b + 1]) ++b;
-    if ((int)blockIdx.x >= cta0[n]) return;
-    sr_main_run<ST, AT, 1, true>(args[b], blockIdx.x - cta0[b], cta0[b + 1] - cta0[b], smem);
 }
 
 // correlator scatter for classes of more states than shared memory holds:
@@ -899,22 +731,12 @@ __global__ void k_axpy_to64(double* x, const VT* d, double scale, int64_t n) {
 // ---------------------------------------------------------------------------
 // explicit instantiations used by the host side
 // ---------------------------------------------------------------------------
-template __global__ void k_sr_main<double, double, 1, true>(MainArgs<double>);
-
-template __global__ void k_sr_main<double, double, 2, true>(MainArgs<double>);
-template __global__ void k_sr_main<double, double, 4, true>(MainArgs<double>);
-template __global__ void k_sr_main<double, double, 2, false>(MainArgs<double>);
-template __global__ void k_sr_main<float, double, 1, true>(MainArgs<double>);
-template __global__ void k_sr_main<float, double, 2, true>(MainArgs<double>);
-template __global__ void k_sr_main<float, double, 4, true>(MainArgs<double>);
-template __global__ void k_sr_main<float, double, 2, false>(MainArgs<double>);
-template __global__ void k_sr_main<float, float, 1, true>(MainArgs<float>);
-template __global__ void k_sr_main<float, float, 2, true>(MainArgs<float>);
-template __global__ void k_sr_main<float, float, 4, true>(MainArgs<float>);
-template __global__ void k_sr_main<__nv_bfloat16, double, 2, false>(MainArgs<double>);
-template __global__ void k_sr_main<__nv_bfloat16, float, 1, true>(MainArgs<float>);
-template __global__ void k_sr_main<__nv_bfloat16, float, 2, true>(MainArgs<float>);
-template __global__ void k_sr_main<__nv_bfloat16, float, 4, true>(MainArgs<float>);
+template __global__ void k_sr_main<float, 1>(MainArgs<float>);
+template __global__ void k_sr_main<float, 2>(MainArgs<float>);
+template __global__ void k_sr_main<float, 4>(MainArgs<float>);
+template __global__ void k_sr_main<__nv_bfloat16, 1>(MainArgs<float>);
+template __global__ void k_sr_main<__nv_bfloat16, 2>(MainArgs<float>);
+template __global__ void k_sr_main<__nv_bfloat16, 4>(MainArgs<float>);
 template __global__ void k_corr_scatter_global<double, 1>(CorrArgs<double>);
 template __global__ void k_corr_scatter_global<double, 2>(CorrArgs<double>);
 template __global__ void k_corr_scatter_global<double, 4>(CorrArgs<double>);
@@ -959,25 +781,5 @@ template __global__ void k_cg_fxrp<float>(CgFusedArgs<float>, const float*, doub
 template __global__ void k_cg_fxrp1<float>(CgFusedArgs<float>, const float*, double*, int*, int);
 template __global__ void k_axpy_to64<float>(double*, const float*, double, int64_t);
 template __global__ void k_axpy_to64<double>(double*, const double*, double, int64_t);
-
-
-// launch of the batched generic pass from the unit that defines it (store_bytes
-// 8: FP64 store, 4: FP32 store; FP64 accumulation)
-cudaError_t launch_sr_main_batch(int store_bytes, int blocks, size_t smem, cudaStream_t st,
-                                 const MainArgs<double>* args, const int* cta0, int n) {
-    cudaError_t e;
-    if (store_bytes == 8) {
-        e = cudaFuncSetAttribute(k_sr_main_batch<double, double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem);
-        if (e != cudaSuccess) return e;
-        k_sr_main_batch<double, double><<<blocks, 512, smem, st>>>(args, cta0, n);
-    } else {
-        e = cudaFuncSetAttribute(k_sr_main_batch<float, double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem);
-        if (e != cudaSuccess) return e;
-        k_sr_main_batch<float, double><<<blocks, 512, smem, st>>>(args, cta0, n);
-    }
-    return cudaGetLastError();
-}
 
 }  // namespace vmc
