@@ -1234,7 +1234,7 @@ static int launch_pass(vmc_ctx* h, const void* s_pf, int store_bytes, int K, boo
     vmc_ctx::PassPlan* L;
     int rc = plan_pass(h, K, gather, &L);
     if (rc) return rc;
-    const int64_t need = (h->n_s + pass_warps(K) - 1) / pass_warps(K);
+    const int64_t need = (h->n_s + 3) / 4;   // a few samples per CTA keep small sets spread over the SMs
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(h->nsm, need));
     if ((size_t)grid * h->npf * K * sizeof(double) > h->pfpart_bytes) return VMC_ERR_UNSUPPORTED;
     vmc_ctx::PassRec rec{};

@@ -101,7 +101,7 @@ struct LogPsiArgs {
     double* out;
 };
 
-template <typename R> __global__ void __launch_bounds__(128, 4) k_walkers(SampleArgs a);
+template <typename R> __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 5 : 4) k_walkers(SampleArgs a);
 cudaError_t launch_walkers_batch(bool fp64, int blocks, int threads, size_t smem, cudaStream_t st,
                                  const SampleArgs* args, const int* wstart, int n, size_t warp_bytes);
 __global__ void k_logpsi(LogPsiArgs a);

@@ -71,12 +71,14 @@ struct PlainAcc {
     using Elem = double;   // a table or image entry
     static __device__ __forceinline__ Elem make(double v) { return v; }
     static __device__ __forceinline__ double value(Elem v) { return v; }
+    static __device__ __forceinline__ void sum(Elem& s, Elem v) { s += v; }
     template <typename W> static __device__ __forceinline__ void add(Elem& s, W w, Elem v) { s = fma(widen(w), v, s); }
 };
 struct PairAcc {
     using Elem = float2;
     static __device__ __forceinline__ Elem make(double v) { return ff_split(v); }
     static __device__ __forceinline__ double value(Elem v) { return (double)v.x + (double)v.y; }
+    static __device__ __forceinline__ void sum(Elem& s, Elem v) { ff_add(s.x, s.y, v.x, v.y); }
     static __device__ __forceinline__ void add(Elem& s, float w, Elem v) {
         const float p = __fmul_rn(w, v.x);
         ff_add(s.x, s.y, p, fmaf(w, v.y, fmaf(w, v.x, -p)));
@@ -220,9 +222,9 @@ __device__ void pass_run(const PassArgs& a, int cta, int ncta, unsigned char* sm
     __syncthreads();
     double* dst = a.pf_partial + (size_t)cta * npf * K;
     for (int i = threadIdx.x; i < npf * K; i += blockDim.x) {
-        double x = 0.0;
-        for (int k = 0; k < ni; ++k) x += A::value(img[(size_t)k * npf * K + i]);
-        dst[i] = x;
+        E x = img[i];
+        for (int k = 1; k < ni; ++k) A::sum(x, img[(size_t)k * npf * K + i]);
+        dst[i] = A::value(x);
     }
 }
 

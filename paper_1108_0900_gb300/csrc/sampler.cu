@@ -410,7 +410,7 @@ __device__ void walker_run(const SampleArgs& a, int w, unsigned char* base) {
 }
 
 template <typename R>
-__global__ void __launch_bounds__(128, 4) k_walkers(SampleArgs a) {
+__global__ void __launch_bounds__(128, sizeof(R) == 4 ? 5 : 4) k_walkers(SampleArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int wid = threadIdx.x >> 5;
     const int w = blockIdx.x * (blockDim.x >> 5) + wid;
@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(128, 4) k_walkers(SampleArgs a) {
 // walker g - wstart[b] of problem b, wstart[b] <= g < wstart[b + 1]; every
 // warp has warp_bytes of shared memory (the largest of the problems').
 template <typename R>
-__global__ void __launch_bounds__(128, 4) k_walkers_batch(const SampleArgs* __restrict__ args,
+__global__ void __launch_bounds__(128, sizeof(R) == 4 ? 5 : 4) k_walkers_batch(const SampleArgs* __restrict__ args,
                                                           const int* __restrict__ wstart, int n,
                                                           size_t warp_bytes) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
