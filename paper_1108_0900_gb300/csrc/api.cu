@@ -176,7 +176,14 @@ struct vmc_ctx {
     std::vector<double> lm_L, lm_R;
     double *d_lmL64 = nullptr, *d_lmR64 = nullptr, *d_lmXt = nullptr, *d_lmxc = nullptr;
     float *d_lmL32 = nullptr, *d_lmR32 = nullptr;
-    int *d_lmLptr = nullptr, *d_lmLidx = nullptr, *d_lmRptr = nullptr, *d_lmRidx = nullptr;
+    int *d_lmLcnt = nullptr, *d_lmLmu = nullptr, *d_lmRptr = nullptr, *d_lmRidx = nullptr;
+    uint8_t* d_lm_need = nullptr;      // moves between sites that some factor holds
+    bool lm_dense = false;
+    std::vector<int> site_cptr, site_corr;    // correlators on every site
+    std::vector<uint32_t> corr_site_w;        // [ncorr][ns] 4^j, 0 if absent
+    int lm_nentry = 0, lm_max_list = 0;
+    int2* d_lm_entries = nullptr;
+    uint64_t* d_lm_common = nullptr;
     // Davidson workspace: basis V and its images (column-major, ld = lm_ld),
     // work vectors, dot partials
     double* d_bcg = nullptr;   // block CG: Gram partials, reduced Gram, alpha, beta
@@ -332,6 +339,9 @@ extern "C" int vmc_create(const vmc_lattice* lat, const vmc_hamiltonian* ham, co
         for (auto& pr : memb[s]) { scorr.push_back(pr.first); sw.push_back(pr.second); }
         scptr[s + 1] = (int)scorr.size();
     }
+    h->site_cptr = scptr;
+    h->site_corr = scorr;
+    h->corr_site_w = csw;
     // hopping lists (each bond hops both ways; repeated bonds repeat)
     std::vector<std::vector<std::pair<int, double>>> nb(ns);
     for (int b = 0; b < lat->n_bonds; ++b) {
@@ -2555,42 +2565,70 @@ extern "C" int sr_local_product(vmc_handle h, const double* v, double* out, int 
 // ---------------------------------------------------------------------------
 static int lm_ensure(vmc_ctx* h) {
     if (h->d_lmL64) return VMC_OK;
-    // the factors as sparse matrices: nonzeros of each L^mu (R^mu) in row order
-    const size_t n2 = (size_t)h->ns * h->ns;
-    std::vector<int> ptr[2], idx[2];
-    std::vector<double> val[2];
-    for (int side = 0; side < 2; ++side) {
-        const std::vector<double>& F = side == 0 ? h->lm_L : h->lm_R;
-        ptr[side].push_back(0);
-        for (int mu = 0; mu < h->lm_nmu; ++mu) {
-            for (size_t t = 0; t < n2; ++t) {
-                const double v = F[(size_t)mu * n2 + t];
-                if (v != 0.0) { idx[side].push_back((int)t); val[side].push_back(v); }
+    // the factors as sparse matrices: the nonzeros of each R^mu in row order; of
+    // the L^mu, entry by entry, [position in the entry's list][entry]
+    const int ns = h->ns;
+    const size_t n2 = (size_t)ns * ns;
+    std::vector<int> ptr(1, 0), idx, cnt(n2, 0);
+    std::vector<double> val;
+    std::vector<uint8_t> need(n2, 0);
+    for (int mu = 0; mu < h->lm_nmu; ++mu) {
+        for (size_t t = 0; t < n2; ++t) {
+            const double v = h->lm_R[(size_t)mu * n2 + t];
+            if (v != 0.0) {
+                idx.push_back((int)t);
+                val.push_back(v);
+                need[t] = 1;                                  // y of the move i -> j
             }
-            ptr[side].push_back((int)idx[side].size());
+            if (h->lm_L[(size_t)mu * n2 + t] != 0.0) {
+                ++cnt[t];
+                need[(t % ns) * ns + t / ns] = 1;             // z_ij is met by the move j -> i
+            }
+        }
+        ptr.push_back((int)idx.size());
+    }
+    const int lmax = std::max(1, *std::max_element(cnt.begin(), cnt.end()));
+    std::vector<int> lmu(n2 * lmax, 0), at(n2, 0);
+    std::vector<double> lval(n2 * lmax, 0.0);
+    for (int mu = 0; mu < h->lm_nmu; ++mu)
+        for (size_t t = 0; t < n2; ++t) {
+            const double v = h->lm_L[(size_t)mu * n2 + t];
+            if (v == 0.0) continue;
+            lmu[at[t] * n2 + t] = mu;
+            lval[at[t]++ * n2 + t] = v;
+        }
+    int needed = 0;
+    for (int i = 0; i < ns; ++i)
+        for (int j = 0; j < ns; ++j) needed += i != j && need[(size_t)i * ns + j];
+    h->lm_dense = 2 * needed > ns * (ns - 1);
+    // single-toggle table entries and the correlators that two sites share
+    h->lm_nentry = (int)h->site_corr.size();
+    std::vector<int2> en((size_t)2 * h->lm_nentry);
+    std::vector<uint64_t> common(n2, 0);
+    for (int s = 0; s < ns; ++s) {
+        const int b = h->site_cptr[s], len = h->site_cptr[s + 1] - b;
+        h->lm_max_list = std::max(h->lm_max_list, len);
+        for (int e = 0; e < len; ++e) {
+            for (int spin = 0; spin < 2; ++spin) en[(size_t)2 * b + spin * len + e] = make_int2(b + e, s << 1 | spin);
+            for (int t = 0; t < ns; ++t)
+                if (t != s && e < 64 && h->corr_site_w[(size_t)h->site_corr[b + e] * ns + t]) common[(size_t)s * ns + t] |= 1ull << e;
         }
     }
-    std::vector<float> L32(val[0].begin(), val[0].end()), R32(val[1].begin(), val[1].end());
-    VCK(h->alloc(&h->d_lmL64, val[0].size()));
-    VCK(h->alloc(&h->d_lmR64, val[1].size()));
-    VCK(h->alloc(&h->d_lmL32, val[0].size()));
-    VCK(h->alloc(&h->d_lmR32, val[1].size()));
-    VCK(h->alloc(&h->d_lmLptr, ptr[0].size()));
-    VCK(h->alloc(&h->d_lmRptr, ptr[1].size()));
-    VCK(h->alloc(&h->d_lmLidx, idx[0].size()));
-    VCK(h->alloc(&h->d_lmRidx, idx[1].size()));
+    std::vector<float> L32(lval.begin(), lval.end()), R32(val.begin(), val.end());
+    auto up = [&](auto** d, const auto& v) -> int {
+        VCK(h->alloc(d, std::max<size_t>(v.size(), 1)));
+        if (!v.empty()) VCK(cudaMemcpy(*d, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice));
+        return VMC_OK;
+    };
+    int rc;
+    if ((rc = up(&h->d_lmR64, val)) || (rc = up(&h->d_lmL32, L32)) || (rc = up(&h->d_lmR32, R32)) ||
+        (rc = up(&h->d_lmLcnt, cnt)) || (rc = up(&h->d_lmLmu, lmu)) || (rc = up(&h->d_lmRptr, ptr)) ||
+        (rc = up(&h->d_lmRidx, idx)) || (rc = up(&h->d_lm_need, need)) || (rc = up(&h->d_lm_entries, en)) ||
+        (rc = up(&h->d_lm_common, common)))
+        return rc;
     VCK(h->alloc(&h->d_lmXt, (size_t)h->M * h->M));
     VCK(h->alloc(&h->d_lmxc, (size_t)std::max<int64_t>(h->ncp, 1)));
-    auto up = [](void* d, const void* s, size_t b) { return b ? cudaMemcpy(d, s, b, cudaMemcpyHostToDevice) : cudaSuccess; };
-    VCK(up(h->d_lmL64, val[0].data(), val[0].size() * sizeof(double)));
-    VCK(up(h->d_lmR64, val[1].data(), val[1].size() * sizeof(double)));
-    VCK(up(h->d_lmL32, L32.data(), L32.size() * sizeof(float)));
-    VCK(up(h->d_lmR32, R32.data(), R32.size() * sizeof(float)));
-    VCK(up(h->d_lmLptr, ptr[0].data(), ptr[0].size() * sizeof(int)));
-    VCK(up(h->d_lmRptr, ptr[1].data(), ptr[1].size() * sizeof(int)));
-    VCK(up(h->d_lmLidx, idx[0].data(), idx[0].size() * sizeof(int)));
-    VCK(up(h->d_lmRidx, idx[1].data(), idx[1].size() * sizeof(int)));
-    return VMC_OK;
+    return up(&h->d_lmL64, lval);   // last: it marks the tables as there
 }
 
 template <typename R>
@@ -2607,26 +2645,34 @@ static int lm_launch(vmc_ctx* h, const double* x, double* Hx, double* Sx, const 
     a.s_occ = h->d_socc; a.Nst = h->Nst;
     a.s_cidx = h->d_cidx; a.ncst = h->ncst;
     a.pf = pf; a.Pst = h->Pst;
-    a.x = x; a.Xt = Xt; a.xc = xc;
+    a.x = x; a.Xt = Xt; a.xc = xc; a.invC = h->d_invC64;
     a.n_mu = h->lm_nmu; a.c0 = h->lm_c0;
-    a.Lptr = h->d_lmLptr; a.Lidx = h->d_lmLidx; a.Lval = Lf;
+    a.Lcnt = h->d_lmLcnt; a.Lmu = h->d_lmLmu; a.Lval = Lf;
     a.Rptr = h->d_lmRptr; a.Ridx = h->d_lmRidx; a.Rval = Rf;
+    a.need = h->d_lm_need; a.dense = h->lm_dense ? 1 : 0;
+    a.pairs = h->max_csites <= 2 ? 1 : 0;
+    a.nentry = h->lm_nentry; a.entries = h->d_lm_entries; a.common = h->d_lm_common;
     a.inv_n = 1.0 / (double)h->n_s;
     a.Hx = Hx; a.Sx = Sx;
-    a.XS = h->N + 1; a.GS = h->N + 1;
-    a.warp_bytes = (int)lm_warp_bytes(h->N, h->M, h->ns, h->lm_nmu, h->ncorr, (int)sizeof(R));
-    if ((size_t)a.warp_bytes > h->smem_optin) {
+    // the workspace of one sample; the single-toggle table where it fits beside it
+    auto layout = [&](bool tables) {
+        return lm_layout(h->ns, h->nu, h->nd, h->lm_nmu, h->ncorr, h->lm_nentry, (int)sizeof(R), tables);
+    };
+    a.L = layout(true);
+    a.tables = (size_t)a.L.bytes + 64 <= h->smem_optin && h->lm_max_list <= 64;
+    if (!a.tables) a.L = layout(false);
+    const size_t smem = (size_t)a.L.bytes;
+    if (smem + 64 > h->smem_optin) {
         set_err("linear-method product: per-sample workspace exceeds shared memory");
         return VMC_ERR_UNSUPPORTED;
     }
-    const int wpb = (int)std::min<size_t>(8, h->smem_optin / (size_t)a.warp_bytes);
-    const size_t smem = (size_t)wpb * a.warp_bytes;
+    // a CTA per sample; eight warps where shared memory leaves few CTAs per SM
+    const int threads = smem > 48 * 1024 ? 256 : 128;
     VCK(cudaFuncSetAttribute(k_lm_apply<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
-    VCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lm_apply<R>, 32 * wpb, smem));
-    const int64_t need = (h->n_s + wpb - 1) / wpb;
-    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)h->nsm * std::max(per_sm, 1)));
-    k_lm_apply<R><<<grid, 32 * wpb, smem, st>>>(a);
+    VCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lm_apply<R>, threads, smem));
+    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(h->n_s, (int64_t)h->nsm * std::max(per_sm, 1)));
+    k_lm_apply<R><<<grid, threads, smem, st>>>(a);
     h->n_launch++;
     VCK(cudaGetLastError());
     return VMC_OK;

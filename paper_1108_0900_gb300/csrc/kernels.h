@@ -413,8 +413,16 @@ __global__ void __launch_bounds__(256) k_sv_finish(SortedArgs a, const float* pf
 // accelerated linear method (Sec. II.B): Eq. 10 products with the basis
 // {Psi, Psi^1 .. Psi^nv} from a stored sample set (lm.cu)
 // ---------------------------------------------------------------------------
+// shared memory of one sample: elements of R from the start, then bytes
+struct LmLayout {
+    int X, G, Xo, Pm, D, Y, w, cold, rcm, fr, fx;
+    int ev_bytes, cidx_bytes, occ_bytes, bytes;
+};
+LmLayout lm_layout(int ns, int nu, int nd, int n_mu, int ncorr, int nentry, int elem, bool tables);
+
 struct LmArgs {
     DevProblem pb;
+    LmLayout L;
     int64_t n_s;
     const uint8_t* s_occ;   // [n_s][Nst] ascending occupied spin orbitals
     int Nst;
@@ -425,21 +433,26 @@ struct LmArgs {
     const double* x;        // [nv + 1]: x_0 then the parameter block
     const void* Xt;         // [M][M] antisymmetric matrix of the pairing part of x (R)
     const void* xc;         // [ncp] x_k / C_k for the correlator part of x (R)
+    const double* invC;     // [ncp] 1 / C_k
     int n_mu;               // factor pairs of Eq. 9, each a sparse ns x ns matrix:
-    const int* Lptr;        // [n_mu + 1] rows of the nonzeros of L^mu
-    const int* Lidx;        // i ns + j of each nonzero
-    const void* Lval;       // its value (R)
-    const int* Rptr;        // the same for R^mu
-    const int* Ridx;
-    const void* Rval;
+    const int* Lcnt;        // [ns ns] factors L^mu with a nonzero at the entry,
+    const int* Lmu;         // [.][ns ns] which (ascending)
+    const void* Lval;       // and their values (R)
+    const int* Rptr;        // [n_mu + 1] rows of the nonzeros of R^mu
+    const int* Ridx;        // i ns + j of each nonzero
+    const void* Rval;       // its value (R)
+    const uint8_t* need;    // [ns][ns] some factor holds the move from one site to the other
+    int dense;              // most moves are needed
+    int pairs;              // correlators of at most two sites
+    int tables;             // the single-toggle table fits (and site lists of at most 64 correlators)
+    int nentry;             // (site, correlator) memberships
+    const int2* entries;    // [2 nentry] of each table entry: membership, site << 1 | spin
+    const uint64_t* common; // [ns][ns] the correlators on the first site that hold the second too
     double c0;
     double inv_n;
     double* Hx;             // [nv + 1], accumulated (zeroed by the caller)
     double* Sx;             // [nv + 1] or null
-    int XS, GS;             // row strides of the per-warp matrices
-    int warp_bytes;
 };
-size_t lm_warp_bytes(int N, int M, int ns, int n_mu, int ncorr, int elem);
 template <typename R> __global__ void k_lm_prep(DevProblem pb, const double* x, R* Xt, R* xc);
 template <typename R> __global__ void k_lm_apply(LmArgs a);
 template <typename R> __global__ void k_lm_diag(LmArgs a, double* d);
