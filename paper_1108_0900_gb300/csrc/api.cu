@@ -660,7 +660,7 @@ extern "C" int vmc_create(const vmc_lattice* lat, const vmc_hamiltonian* ham, co
     pb.eri_nk = (int)round_up(ns, 4);
     pb.dexc = h->d_dexc;
     pb.max_csites = h->max_csites;
-    pb.C64 = h->d_C64; pb.C32 = h->d_C32; pb.F64 = h->d_F64; pb.F32 = h->d_F32;
+    pb.C64 = h->d_C64; pb.iC64 = h->d_invC64; pb.C32 = h->d_C32; pb.F64 = h->d_F64; pb.F32 = h->d_F32;
     pb.pairtab = h->d_pairtab; pb.rowbase = h->d_rowbase;
     *out = h;
     return VMC_OK;
@@ -743,13 +743,14 @@ extern "C" int vmc_get_params(vmc_handle h, double* C, double* f, void* stream) 
 }
 
 static int check_configs(const vmc_ctx* h, const uint8_t* occ, int64_t n) {
+    // no early exit inside a configuration: the loop vectorises
     for (int64_t w = 0; w < n; ++w) {
         const uint8_t* o = occ + w * h->N;
-        for (int a = 0; a < h->N; ++a) {
-            if (o[a] >= h->M) return VMC_ERR_INVALID_ARG;
-            if (a > 0 && o[a] <= o[a - 1]) return VMC_ERR_INVALID_ARG;
-            if ((a < h->nu) != (o[a] < h->ns)) return VMC_ERR_INVALID_ARG;
-        }
+        unsigned bad = 0;
+        for (int a = 0; a < h->nu; ++a) bad |= o[a] >= h->ns;
+        for (int a = h->nu; a < h->N; ++a) bad |= (o[a] < h->ns) | (o[a] >= h->M);
+        for (int a = 1; a < h->N; ++a) bad |= o[a] <= o[a - 1];
+        if (bad) return VMC_ERR_INVALID_ARG;
     }
     return VMC_OK;
 }
@@ -807,6 +808,20 @@ static size_t prep_walkers(vmc_ctx* h, SampleArgs& a, bool fp64) {
 }
 
 static int launch_walkers(vmc_ctx* h, SampleArgs& a, bool fp64, cudaStream_t st) {
+    if (fp64 && a.props_per_sweep == 0) {
+        // given configurations, FP64 from scratch: four warps (samples) per CTA, or fewer
+        int warps = 4;
+        while (warps > 1 && measure64_smem(h->N, h->P, h->ncorr, warps) > h->smem_optin) warps /= 2;
+        const size_t smem = measure64_smem(h->N, h->P, h->ncorr, warps);
+        if (smem > h->smem_optin) return VMC_ERR_UNSUPPORTED;
+        a.status = h->d_status;
+        a.pb = h->pb;
+        VCK(cudaFuncSetAttribute(k_measure64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        k_measure64<<<(unsigned)((a.n_walkers + warps - 1) / warps), 32 * warps, smem, st>>>(a, h->d_fulltab);
+        h->n_launch++;
+        VCK(cudaGetLastError());
+        return VMC_OK;
+    }
     const size_t wb = prep_walkers(h, a, fp64);
     int wpb = (int)std::min<size_t>(4, h->smem_optin / wb);
     if (wpb < 1) return VMC_ERR_UNSUPPORTED;
@@ -1150,11 +1165,10 @@ extern "C" int vmc_logpsi(vmc_handle h, double* out, void* stream) {
     a.n_s = h->n_s;
     a.s_occ = h->d_socc; a.Nst = h->Nst;
     a.s_cidx = h->d_cidx; a.ncst = h->ncst;
-    a.XS = h->N + 1;
-    a.warp_bytes = round_up((size_t)h->N * a.XS * 8 + 2 * (size_t)a.XS * 8, 16);
-    int wpb = 4;
-    size_t smem = a.warp_bytes * wpb;
+    a.fulltab = h->d_fulltab;
     a.out = out;
+    const int wpb = 4;
+    const size_t smem = measure64_smem(h->N, h->P, 0, wpb);
     VCK(cudaFuncSetAttribute(k_logpsi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     k_logpsi<<<(unsigned)((h->n_s + wpb - 1) / wpb), 32 * wpb, smem, st>>>(a); h->n_launch++;
     VCK(cudaGetLastError());

@@ -133,6 +133,7 @@ struct DevProblem {
     const uint16_t* dexc;
     // parameters
     const double* C64;
+    const double* iC64;        // 1 / C
     const float* C32;
     const double* F64;         // M x M antisymmetric
     const float* F32;

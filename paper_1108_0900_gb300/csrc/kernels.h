@@ -96,15 +96,17 @@ struct LogPsiArgs {
     int Nst;
     const cstate_t* s_cidx;
     int ncst;
-    int XS;
-    size_t warp_bytes;
+    const uint32_t* fulltab;   // as PassArgs
     double* out;
 };
 
 template <typename R> __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 5 : 4) k_walkers(SampleArgs a);
 cudaError_t launch_walkers_batch(bool fp64, int blocks, int threads, size_t smem, cudaStream_t st,
                                  const SampleArgs* args, const int* wstart, int n, size_t warp_bytes);
-__global__ void k_logpsi(LogPsiArgs a);
+// FP64 evaluation of given configurations from scratch (measure64.cu)
+size_t measure64_smem(int N, int P, int ncorr, int warps);
+__global__ void __launch_bounds__(128) k_measure64(SampleArgs a, const uint32_t* fulltab);
+__global__ void __launch_bounds__(128) k_logpsi(LogPsiArgs a);
 
 // ---------------------------------------------------------------------------
 // SR kernels

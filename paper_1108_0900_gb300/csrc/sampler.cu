@@ -372,29 +372,14 @@ __device__ void walker_run(const SampleArgs& a, int w, unsigned char* base) {
             for (int t = lane; t < N * N; t += 32) dst[t] = X[(t / N) * XS + t % N];
             for (int i = lane; i < N; i += 32) a.s_pos[s * a.Nst + i] = pos_orb[i];
         }
-        if (a.bgrad) {
-            // adjoint: grad += w_s O(n_s)
-            double ws = a.bw[s];
-            for (int c = lane; c < pb.ncorr; c += 32) {
-                int64_t k = pb.corr_off[c] + cidx[c];
-                atomicAdd(a.bgrad + k, ws / pb.C64[k]);
-            }
-            for (int e = lane; e < pb.P; e += 32) {
-                uint16_t t = pb.pairtab[e];
-                int aa = t & 255, bb = t >> 8;
-                int oa = pos_orb[iv[aa]], ob = pos_orb[iv[bb]];
-                atomicAdd(a.bgrad + pb.ncp + pb.rowbase[oa] + ob, ws * (double)X[iv[bb] * XS + iv[aa]]);
-            }
-        } else {
-            if (a.s_E && pb.ham == 0 && lane == 0) a.s_E[s] = e_lane;
-            if (a.s_lnrun && lane == 0) a.s_lnrun[s] = lnrun;
-            if (a.s_cidx)
-                for (int c = lane; c < pb.ncorr; c += 32) a.s_cidx[s * a.ncst + c] = (cstate_t)cidx[c];
-            for (int e = lane; e < pb.P; e += 32) {
-                uint16_t t = pb.pairtab[e];
-                int aa = t & 255, bb = t >> 8;
-                store_pf<R>(a, s * a.Pst + e, X[iv[bb] * XS + iv[aa]]);
-            }
+        if (a.s_E && pb.ham == 0 && lane == 0) a.s_E[s] = e_lane;
+        if (a.s_lnrun && lane == 0) a.s_lnrun[s] = lnrun;
+        if (a.s_cidx)
+            for (int c = lane; c < pb.ncorr; c += 32) a.s_cidx[s * a.ncst + c] = (cstate_t)cidx[c];
+        for (int e = lane; e < pb.P; e += 32) {
+            uint16_t t = pb.pairtab[e];
+            int aa = t & 255, bb = t >> 8;
+            store_pf<R>(a, s * a.Pst + e, X[iv[bb] * XS + iv[aa]]);
         }
         __syncwarp();
     }
@@ -432,78 +417,6 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 5 : 4) k_walkers_batch(c
     int b = 0;
     while (b + 1 < n && g >= wstart[b + 1]) ++b;
     walker_run<R>(args[b], g - wstart[b], smem_raw + (size_t)wid * warp_bytes);
-}
-
-// ln|Pf(F[occ, occ])| + sum_c ln|C_c| per sample, FP64 Parlett-Reid with
-// pivoting (the pfaffian reduction cited in Sec. II.C), one warp per sample.
-__global__ void k_logpsi(LogPsiArgs a) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const DevProblem& pb = a.pb;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t s = (int64_t)blockIdx.x * (blockDim.x >> 5) + wid;
-    if (s >= a.n_s) return;
-    const int N = pb.N, XS = a.XS;
-    double* A = (double*)(smem_raw + (size_t)wid * a.warp_bytes);
-    double* tau = A + N * XS;
-    double* colk1 = tau + XS;
-    const uint8_t* occ = a.s_occ + s * a.Nst;
-    for (int i = 0; i < N; ++i)
-        for (int j = lane; j < N; j += 32) A[i * XS + j] = __ldg(pb.F64 + occ[i] * pb.M + occ[j]);
-    __syncwarp();
-    double logabs = 0.0;
-    int sign = 1;
-    for (int k = 0; k + 1 < N; k += 2) {
-        double best = -1.0;
-        int bi = N;
-        for (int i = k + 1 + lane; i < N; i += 32) {
-            double v = fabs(A[i * XS + k]);
-            if (v > best) { best = v; bi = i; }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            double ob = __shfl_xor_sync(VMC_FULL_MASK, best, o);
-            int oi = __shfl_xor_sync(VMC_FULL_MASK, bi, o);
-            if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-        }
-        if (!(best > 0.0)) { sign = 0; break; }
-        if (bi != k + 1) {
-            for (int j = lane; j < N; j += 32) {
-                double t = A[(k + 1) * XS + j];
-                A[(k + 1) * XS + j] = A[bi * XS + j];
-                A[bi * XS + j] = t;
-            }
-            __syncwarp();
-            for (int i = lane; i < N; i += 32) {
-                double t = A[i * XS + k + 1];
-                A[i * XS + k + 1] = A[i * XS + bi];
-                A[i * XS + bi] = t;
-            }
-            sign = -sign;
-        }
-        __syncwarp();
-        double piv = A[k * XS + k + 1];
-        if (piv < 0) sign = -sign;
-        logabs += log(fabs(piv));
-        for (int i = k + 2 + lane; i < N; i += 32) {
-            tau[i] = A[k * XS + i] / piv;
-            colk1[i] = A[i * XS + k + 1];
-        }
-        __syncwarp();
-        for (int j = k + 2 + lane; j < N; j += 32) {
-            double tj = tau[j], cj = colk1[j];
-            for (int i = k + 2; i < N; ++i) A[i * XS + j] += tau[i] * cj - colk1[i] * tj;
-        }
-        __syncwarp();
-    }
-    // correlators
-    const cstate_t* ci = a.s_cidx + s * a.ncst;
-    double lc = 0.0;
-    for (int c = lane; c < pb.ncorr; c += 32) {
-        double v = pb.C64[pb.corr_off[c] + ci[c]];
-        lc += log(fabs(v));
-    }
-    lc = warp_sum(lc);
-    if (lane == 0) a.out[s] = sign == 0 ? -INFINITY : logabs + lc;
 }
 
 template __global__ void k_walkers<float>(SampleArgs);
