@@ -46,7 +46,14 @@ struct vmc_ctx {
     int64_t ncap = 0, n_s = 0;
     int wprec = VMC_FP64, keep64 = 1, keeplow = 0, refresh_every = 0, fp64_refresh = 0;
     int ham = 0;
-    int maxd = 1;
+    int maxd = 1, mind = 1 << 30;   // states of the largest and smallest correlator
+    std::vector<int> dims;          // and of every one
+    int mid_d(int most) const {     // of the largest with at most `most`
+        int d = 0;
+        for (int x : dims)
+            if (x <= most) d = std::max(d, x);
+        return d;
+    }
     int max_csites = 0;          // sites of the largest correlator
     struct PassPlan {            // launch shape of a pass with FP64 sums (see plan_pass)
         int ni = 0;              // images per CTA
@@ -292,6 +299,8 @@ extern "C" int vmc_create(const vmc_lattice* lat, const vmc_hamiltonian* ham, co
         }
         cptr[c + 1] = (int)csites.size();
         h->maxd = std::max(h->maxd, 1 << (2 * m));
+        h->mind = std::min(h->mind, 1 << (2 * m));
+        h->dims.push_back(1 << (2 * m));
     }
     // classes: correlators of one class share one parameter block; blocks in
     // class order, corr_off[c] = first parameter of c's block
@@ -799,7 +808,8 @@ static size_t prep_walkers(vmc_ctx* h, SampleArgs& a, bool fp64) {
     a.XS = (h->N + 2) & ~1;   // even (the rank-2 update moves column pairs), N + 1 or N + 2
     a.ncorr_pad = (int)round_up(std::max(h->ncorr, 1), 4);
     const size_t rsz = fp64 ? 8 : 4;
-    size_t wb = (size_t)h->N * a.XS * rsz + 3 * (size_t)a.XS * rsz;
+    // (the last two vectors also hold the local energy's queue of 32 words)
+    size_t wb = (size_t)h->N * a.XS * rsz + (size_t)a.XS * rsz + std::max<size_t>(2 * (size_t)a.XS * rsz, 128);
     wb = wb + 64 + (size_t)a.ncorr_pad * 4 + 64 + 128;
     wb = round_up(wb, 16);
     a.warp_bytes = wb;
@@ -1403,6 +1413,9 @@ static int launch_corr(vmc_ctx* h, const AT* T, const int* stop, cudaStream_t st
         VCK(cudaGetLastError());
         return VMC_OK;
     }
+    // a histogram per thread for classes of at most 64 values
+    if (h->mind * K <= 64) smem = std::max(smem, (size_t)h->mid_d(64 / K) * K * (256 + 1) * sizeof(AT));
+    a.cap = (int)(smem / sizeof(AT));
     auto kern = k_corr_scatter<AT, K>;
     VCK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     kern<<<h->n_units * kCorrCluster, 256, smem, st>>>(a); h->n_launch++;

@@ -169,6 +169,7 @@ struct CorrArgs {
     const AT* T;            // [n_s][K]
     AT* corr_raw;           // [ncp][K] sum over samples of t_s per state (zeroed by the caller)
     const int4* units;      // cluster work units (class, first, end into class_inst)
+    int cap;                // elements of the kernel's shared memory
     const int* stop;
 };
 
