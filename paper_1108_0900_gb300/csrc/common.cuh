@@ -59,6 +59,18 @@ __device__ __forceinline__ int nth_set_bit64(uint64_t mask, int n) {
     return 32 + __fns(hi, 0, n - cl + 1);
 }
 
+// the same when mask and n are the warp's: every lane looks at one bit
+__device__ __forceinline__ int nth_set_bit_warp(uint64_t mask, int n) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t lo = (uint32_t)mask, hi = (uint32_t)(mask >> 32);
+    const int cl = __popc(lo);
+    const bool low = n < cl;
+    const uint32_t w = low ? lo : hi;
+    const int k = low ? n : n - cl;
+    const uint32_t b = __ballot_sync(VMC_FULL_MASK, ((w >> lane) & 1u) && __popc(w & ((1u << lane) - 1u)) == k);
+    return (low ? 0 : 32) + __ffs(b) - 1;
+}
+
 __device__ __forceinline__ uint32_t mulhi32(uint32_t a, uint32_t b) {
     return (uint32_t)(((uint64_t)a * (uint64_t)b) >> 32);
 }

@@ -29,9 +29,30 @@ struct WarpMem {
 };
 
 
-// ln|x| in the walker's precision (FP32 chains avoid the FP64 pipe)
-__device__ __forceinline__ float log_abs(float x) { return logf(fabsf(x)); }
-__device__ __forceinline__ double log_abs(double x) { return log(fabs(x)); }
+// Running product of the accepted ratios' magnitudes as m 2^e, m in [1, 2): one
+// multiplication per accepted move, and one logarithm per stored sample instead
+// of one per move (an FP64 logarithm is a hundred dependent instructions on a
+// pipe of 16 cycles each: 40 % of an accepted move on small lattices).
+struct LogProduct {
+    double m = 1.0;
+    int e = 0;
+    __device__ __forceinline__ void mul(double x) {
+        m *= fabs(x);
+        const int hi = __double2hiint(m), ex = (hi >> 20) & 0x7ff;
+        if (ex != 0 && ex != 0x7ff) {   // zero, denormal, infinite or NaN: left to the logarithm
+            e += ex - 1023;
+            m = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(m));
+        }
+    }
+    __device__ __forceinline__ double log_value() const { return log(m) + (double)e * 0.69314718055994530942; }
+};
+
+// correlator amplitude ratio C(new) / C(old): FP64 walkers multiply by the stored
+// 1 / C (a division there is a dozen dependent FP64 instructions)
+__device__ __forceinline__ float load_den(const DevProblem& pb, int64_t k, float) { return __ldg(pb.C32 + k); }
+__device__ __forceinline__ double load_den(const DevProblem& pb, int64_t k, double) { return __ldg(pb.iC64 + k); }
+__device__ __forceinline__ float ratio_of(float num, float den) { return num / den; }
+__device__ __forceinline__ double ratio_of(double num, double inv) { return num * inv; }
 
 template <typename R> struct pair_of;
 template <> struct pair_of<float> { using type = float2; };
@@ -51,7 +72,7 @@ __device__ R corr_ratio_warp(const DevProblem& pb, uint32_t* cidx, int p, int q,
         int c = -1, newi = -1;
         if (e < total) {
             newi = corr_entry(pb, cidx, sp, sq, sf, e, &c);
-            if (c >= 0) r = load_C<R>(pb, pb.corr_off[c] + newi) / load_C<R>(pb, pb.corr_off[c] + cidx[c]);
+            if (c >= 0) r = ratio_of(load_C<R>(pb, pb.corr_off[c] + newi), load_den(pb, pb.corr_off[c] + cidx[c], R(0)));
         }
         prod *= warp_prod(r);
         if (commit) {
@@ -59,6 +80,22 @@ __device__ R corr_ratio_warp(const DevProblem& pb, uint32_t* cidx, int p, int q,
             if (c >= 0) cidx[c] = (uint32_t)newi;
             __syncwarp();
         }
+    }
+    return prod;
+}
+
+// the same by one lane, for a hop of its own
+template <typename R>
+__device__ R corr_ratio_hop(const DevProblem& pb, const uint32_t* cidx, int p, int q) {
+    const int ns = pb.ns, sf = p >= ns ? 2 : 1;
+    const int sp = p >= ns ? p - ns : p, sq = q >= ns ? q - ns : q;
+    const int total = (pb.site_cptr[sp + 1] - pb.site_cptr[sp]) + (pb.site_cptr[sq + 1] - pb.site_cptr[sq]);
+    R prod = R(1);
+#pragma unroll 4
+    for (int e = 0; e < total; ++e) {
+        int c;
+        const int newi = corr_entry(pb, cidx, sp, sq, sf, e, &c);
+        if (c >= 0) prod *= ratio_of(load_C<R>(pb, pb.corr_off[c] + newi), load_den(pb, pb.corr_off[c] + cidx[c], R(0)));
     }
     return prod;
 }
@@ -157,7 +194,7 @@ __device__ void walker_run(const SampleArgs& a, int w, unsigned char* base) {
     R* bv = X + N * XS;
     R* yv = bv + XS;
     R* cv = yv + XS;
-    uint8_t* iv = (uint8_t*)(cv + XS);         // 64 positions
+    uint8_t* iv = (uint8_t*)yv + max(2 * XS * (int)sizeof(R), 128);   // 64 positions (yv, cv: also a queue of 32 words)
     uint32_t* cidx = (uint32_t*)(iv + 64);     // ncorr (rounded up to 4)
     uint8_t* pos_orb = (uint8_t*)(cidx + a.ncorr_pad);
     int8_t* orb_pos = (int8_t*)(pos_orb + 64); // 128
@@ -208,7 +245,7 @@ __device__ void walker_run(const SampleArgs& a, int w, unsigned char* base) {
 
     const uint64_t sitemask = (ns == 64) ? ~0ull : ((1ull << ns) - 1ull);
     uint64_t step = a.walker_step ? a.walker_step[w] : 0ull;
-    double lnrun = 0.0;   // ln|Psi| of the chain relative to its start, summed from the accepted ratios
+    LogProduct psi;       // |Psi| of the chain relative to its start, from the accepted ratios
     const uint32_t k0 = (uint32_t)a.seed, k1 = (uint32_t)(a.seed >> 32);
     const int n_sweeps = a.n_burn + a.spw;
     // Philox words of 32 consecutive proposals at once: lane L holds those of
@@ -232,13 +269,13 @@ __device__ void walker_run(const SampleArgs& a, int w, unsigned char* base) {
             r.z = __shfl_sync(VMC_FULL_MASK, rl.z, rsrc);
             ++step;
             int as = (int)mulhi32(r.x, (uint32_t)N);
-            int p = as < nu ? nth_set_bit64(up, as) : ns + nth_set_bit64(dn, as - nu);
+            int p = as < nu ? nth_set_bit_warp(up, as) : ns + nth_set_bit_warp(dn, as - nu);
             int spin = p >= ns;
             uint64_t m = spin ? dn : up;
             int n_empty = ns - __popcll(m);
             if (n_empty <= 0) continue;
             int kk = (int)mulhi32(r.y, (uint32_t)n_empty);
-            int q = spin * ns + nth_set_bit64(~m & sitemask, kk);
+            int q = spin * ns + nth_set_bit_warp(~m & sitemask, kk);
             R u = R(r.z >> 8) * R(1.0 / 16777216.0);
             int ap = orb_pos[p];
             // correlator factor, one membership entry per lane when the two
@@ -253,7 +290,7 @@ __device__ void walker_run(const SampleArgs& a, int w, unsigned char* base) {
                 cnew = corr_entry(pb, cidx, csp, csq, csf, lane, &cc);
                 if (cc >= 0) {
                     cnum = load_C<R>(pb, pb.corr_off[cc] + cnew);
-                    cden = load_C<R>(pb, pb.corr_off[cc] + cidx[cc]);
+                    cden = load_den(pb, pb.corr_off[cc] + cidx[cc], R(0));
                 }
             }
             R acc = R(0);
@@ -263,11 +300,11 @@ __device__ void walker_run(const SampleArgs& a, int w, unsigned char* base) {
                 acc += bj * X[ap * XS + j];
             }
             R rpf = -warp_sum(acc);
-            R rc = cfast ? warp_prod(cnum / cden) : corr_ratio_warp<R>(pb, cidx, p, q, false);
+            R rc = cfast ? warp_prod(ratio_of(cnum, cden)) : corr_ratio_warp<R>(pb, cidx, p, q, false);
             R ratio = rpf * rc;
             bool accept = u < ratio * ratio;
             if (!accept) continue;
-            lnrun += (double)log_abs(ratio);
+            psi.mul((double)ratio);
             __syncwarp();
             {
                 // lane L owns the column pair 2L, 2L + 1 (XS even); X is
@@ -297,13 +334,22 @@ __device__ void walker_run(const SampleArgs& a, int w, unsigned char* base) {
                 __syncwarp();
                 if (own) {
                     // X_ij += (c_i y_j - y_i c_j) / r
-                    for (int i = 0; i < N; ++i) {
-                        const R2 ci = cy[i];
-                        R2* xp = reinterpret_cast<R2*>(X + i * XS + j0);
-                        R2 x = *xp;
-                        x.x = fma(ci.x, yj.x, fma(-ci.y, cj.x, x.x));
-                        x.y = fma(ci.x, yj.y, fma(-ci.y, cj.y, x.y));
-                        *xp = x;
+                    // (four rows' loads ahead of their stores)
+                    for (int i = 0; i < N; i += 4) {
+                        R2 x[4], ci[4];
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) {
+                            const int iv4 = min(i + v, N - 1);
+                            ci[v] = cy[iv4];
+                            x[v] = *reinterpret_cast<const R2*>(X + iv4 * XS + j0);
+                        }
+#pragma unroll
+                        for (int v = 0; v < 4; ++v)
+                            if (i + v < N) {
+                                x[v].x = fma(ci[v].x, yj.x, fma(-ci[v].y, cj.x, x[v].x));
+                                x[v].y = fma(ci[v].x, yj.y, fma(-ci[v].y, cj.y, x[v].y));
+                                *reinterpret_cast<R2*>(X + (i + v) * XS + j0) = x[v];
+                            }
                     }
                 }
             }
@@ -336,26 +382,46 @@ __device__ void walker_run(const SampleArgs& a, int w, unsigned char* base) {
         const int64_t s = (int64_t)w * a.spw + (sw - a.n_burn);
         double e_lane = 0.0;
         if (a.want_energy && pb.ham == 0) {   // the ab initio energy has a pass of its own (abinitio.cu)
-            {
-                for (int i = lane; i < N; i += 32) {
-                    int p = pos_orb[i];
-                    int spin = p >= ns;
-                    int sp = p - spin * ns;
-                    uint64_t m = spin ? dn : up;
-                    for (int k = pb.nbr_ptr[sp]; k < pb.nbr_ptr[sp + 1]; ++k) {
-                        int s2 = pb.nbr_site[k];
-                        if ((m >> s2) & 1ull) continue;
-                        int q = spin * ns + s2;
-                        R d = R(0);
+            // a lane per open hop: (electron, entry of its site's neighbour list)
+            // queue up until 32 are there, so that every lane of the pfaffian row
+            // products and correlator factors works
+            auto hop = [&](uint32_t en) {
+                const int i = (int)(en & 255u), k = (int)(en >> 8), p = pos_orb[i];
+                const int q = (p >= ns) * ns + pb.nbr_site[k];
+                R d = R(0);
 #pragma unroll 8
-                        for (int j = 0; j < N; ++j)
-                            if (j != i) d += load_F<R>(pb, q, pos_orb[j]) * X[i * XS + j];
-                        R rc = corr_ratio_serial<R>(pb, cidx, p, q);
-                        // -t * (Pf ratio = -d) * rc
-                        e_lane += pb.nbr_t[k] * (double)(d * rc);
+                for (int j = 0; j < N; ++j)
+                    if (j != i) d += load_F<R>(pb, q, pos_orb[j]) * X[i * XS + j];
+                R rc = corr_ratio_hop<R>(pb, cidx, p, q);
+                // -t * (Pf ratio = -d) * rc
+                e_lane += pb.nbr_t[k] * (double)(d * rc);
+            };
+            uint32_t* queue = reinterpret_cast<uint32_t*>(yv);   // 32 entries
+            int nq = 0;
+            for (int i = 0; i < N; ++i) {
+                const int p = pos_orb[i], spin = p >= ns, sp = p - spin * ns;
+                const uint64_t m = spin ? dn : up;
+                const int k1 = pb.nbr_ptr[sp + 1];
+                for (int k0 = pb.nbr_ptr[sp]; k0 < k1; k0 += 32) {
+                    const int k = k0 + lane;
+                    const bool open = k < k1 && !((m >> pb.nbr_site[k < k1 ? k : k0]) & 1ull);
+                    const uint32_t b = __ballot_sync(VMC_FULL_MASK, open), en = (uint32_t)i | (uint32_t)k << 8;
+                    const int at = nq + __popc(b & ((1u << lane) - 1u));
+                    if (open && at < 32) queue[at] = en;
+                    nq += __popc(b);
+                    if (nq >= 32) {
+                        __syncwarp();
+                        const uint32_t mine = queue[lane];
+                        __syncwarp();
+                        if (open && at >= 32) queue[at - 32] = en;
+                        nq -= 32;
+                        hop(mine);
                     }
                 }
             }
+            __syncwarp();
+            if (lane < nq) hop(queue[lane]);
+            __syncwarp();
             e_lane = warp_sum(e_lane);
             e_lane += pb.U * (double)__popcll(up & dn);
             if (!isfinite(e_lane) && lane == 0) atomicOr(a.status, ST_NONFINITE);
@@ -373,7 +439,7 @@ __device__ void walker_run(const SampleArgs& a, int w, unsigned char* base) {
             for (int i = lane; i < N; i += 32) a.s_pos[s * a.Nst + i] = pos_orb[i];
         }
         if (a.s_E && pb.ham == 0 && lane == 0) a.s_E[s] = e_lane;
-        if (a.s_lnrun && lane == 0) a.s_lnrun[s] = lnrun;
+        if (a.s_lnrun && lane == 0) a.s_lnrun[s] = psi.log_value();
         if (a.s_cidx)
             for (int c = lane; c < pb.ncorr; c += 32) a.s_cidx[s * a.ncst + c] = (cstate_t)cidx[c];
         for (int e = lane; e < pb.P; e += 32) {
