@@ -57,6 +57,7 @@ struct vmc_ctx {
     int max_csites = 0;          // sites of the largest correlator
     struct PassPlan {            // launch shape of a pass with FP64 sums (see plan_pass)
         int ni = 0;              // images per CTA
+        int nimg = 0;            // entries of an image
         int64_t n_s = -1;        // of the samples that it is for (-1: not planned)
         size_t smem = 0;
     } pass_plan[4];              // one, two, four vectors; the gradient
@@ -148,6 +149,7 @@ struct vmc_ctx {
     double* d_Obar[3] = {nullptr, nullptr, nullptr};
     float* d_Obar32[3] = {nullptr, nullptr, nullptr};   // FP32 copies for the inner solve
     int* d_status = nullptr;
+    bool status_live = false;   // a kernel that may set d_status was given it since the last read_status
     // scratch
     void* d_T = nullptr;
     void* d_pfpart = nullptr;
@@ -220,6 +222,7 @@ struct vmc_ctx {
         if (e == cudaSuccess) { allocs.push_back(q); *p = (T*)q; }
         return e;
     }
+    int* status_word() { status_live = true; return d_status; }
     double* part(int slot) { return d_part + (size_t)slot * kNumPart * kMaxK; }
 };
 
@@ -788,12 +791,18 @@ extern "C" int vmc_get_walkers(vmc_handle h, uint8_t* occ, uint64_t* step, void*
 // ---------------------------------------------------------------------------
 // walker kernels
 // ---------------------------------------------------------------------------
+// waits for the stream; the status word is fetched if a kernel could have set it
 static int read_status(vmc_ctx* h, cudaStream_t st) {
     int s = 0;
+    if (!h->status_live) {
+        VCK(cudaStreamSynchronize(st));
+        return VMC_OK;
+    }
     VCK(cudaMemcpyAsync(h->h_pinned, h->d_status, sizeof(int), cudaMemcpyDeviceToHost, st));
     VCK(cudaStreamSynchronize(st));
     memcpy(&s, h->h_pinned, sizeof(int));
-    VCK(cudaMemsetAsync(h->d_status, 0, sizeof(int), st));
+    h->status_live = false;
+    if (s) VCK(cudaMemsetAsync(h->d_status, 0, sizeof(int), st));
     if (s & ST_BAD_CONFIG) return VMC_ERR_INVALID_ARG;
     if (s & ST_SINGULAR) return VMC_ERR_SINGULAR;
     if (s & ST_NONFINITE) return VMC_ERR_NONFINITE;
@@ -813,7 +822,7 @@ static size_t prep_walkers(vmc_ctx* h, SampleArgs& a, bool fp64) {
     wb = wb + 64 + (size_t)a.ncorr_pad * 4 + 64 + 128;
     wb = round_up(wb, 16);
     a.warp_bytes = wb;
-    a.status = h->d_status;
+    a.status = h->status_word();
     return wb;
 }
 
@@ -824,7 +833,7 @@ static int launch_walkers(vmc_ctx* h, SampleArgs& a, bool fp64, cudaStream_t st)
         while (warps > 1 && measure64_smem(h->N, h->P, h->ncorr, warps) > h->smem_optin) warps /= 2;
         const size_t smem = measure64_smem(h->N, h->P, h->ncorr, warps);
         if (smem > h->smem_optin) return VMC_ERR_UNSUPPORTED;
-        a.status = h->d_status;
+        a.status = h->status_word();
         a.pb = h->pb;
         VCK(cudaFuncSetAttribute(k_measure64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         k_measure64<<<(unsigned)((a.n_walkers + warps - 1) / warps), 32 * warps, smem, st>>>(a, h->d_fulltab);
@@ -889,7 +898,7 @@ static int ab_energy(vmc_ctx* h, bool fp64, int64_t n_s, cudaStream_t st) {
     a.s_cidx = h->d_cidx; a.ncst = h->ncst;
     a.X = h->d_abX;
     a.s_E = h->d_E;
-    a.status = h->d_status;
+    a.status = h->status_word();
     const size_t rest = (size_t)h->N * (h->N | 1) * rsz + (size_t)h->ncorr * 4 + 64 + 3 * 128;
     int nw = kAbThreads / 32;
     AbLayout L = ab_layout(h->ns, h->nu, h->nd, nw);
@@ -1212,9 +1221,10 @@ extern "C" int vmc_logpsi_backward(vmc_handle h, const double* w, double* grad, 
 static int plan_pass(vmc_ctx* h, int K, bool gather, vmc_ctx::PassPlan** out) {
     vmc_ctx::PassPlan& L = h->pass_plan[!gather ? 3 : K == 1 ? 0 : K == 2 ? 1 : 2];
     if (L.n_s != h->n_s) {
+        auto smem = [&](int nimg, int ni) { return pass_smem(h->npf, nimg, h->P, K, gather, ni); };
         int ni = pass_warps(K);
-        while (ni > 1 && pass_smem(h->npf, h->P, K, gather, ni) > h->smem_optin) ni /= 2;
-        if (pass_smem(h->npf, h->P, K, gather, ni) > h->smem_optin) {
+        while (ni > 1 && smem(h->npf, ni) > h->smem_optin) ni /= 2;
+        if (smem(h->npf, ni) > h->smem_optin) {
             set_err("pairing block does not fit in shared memory");
             return VMC_ERR_UNSUPPORTED;
         }
@@ -1222,7 +1232,14 @@ static int plan_pass(vmc_ctx* h, int K, bool gather, vmc_ctx::PassPlan** out) {
         // and added up once per element of the pairing block
         const double per_cta = (double)h->n_s * h->P / h->nsm;
         while (ni > 1 && (double)ni * h->npf > per_cta) ni /= 2;
-        L.smem = pass_smem(h->npf, h->P, K, gather, ni);
+        // correlator blocks of up to four pairing blocks, each one's own, enter the
+        // images where these fit all the same: 4x4 lattice, pair correlators, 4,096
+        // samples, about 1 us more in the pass for a launch of 10.7 us
+        const int64_t all = h->npf + h->ncp;
+        const bool with = h->n_class == h->ncorr && h->ncp > 0 && all <= 4 * (int64_t)h->npf &&
+                          smem((int)all, ni) <= h->smem_optin;
+        L.nimg = with ? (int)all : h->npf;
+        L.smem = smem(L.nimg, ni);
         L.ni = ni;
         L.n_s = h->n_s;
     }
@@ -1242,6 +1259,8 @@ static void pass_args(const vmc_ctx* h, const vmc_ctx::PassPlan& L, int K, const
     a.V = V; a.invC = h->d_invC64; a.T = T;
     a.pf_partial = (double*)h->d_pfpart;
     a.ni = L.ni;
+    a.nimg = L.nimg;
+    if (L.nimg == h->npf && h->ncp > 0) a.clear = h->d_corrraw;
     a.stop = stop;
     // orbitals where an image's owners begin: equal shares of the expected number
     // of pairs (p, q > p) at the sector's mean occupations
@@ -1262,15 +1281,39 @@ static void pass_args(const vmc_ctx* h, const vmc_ctx::PassPlan& L, int K, const
     while (f <= owners) a.bounds[f++] = h->M;
 }
 
-// pass with FP64 sums over the FP64, FP32 or (gradient only) BF16 store
+static void finish_args(const vmc_ctx* h, const vmc_ctx::PassPlan& L, int nblk, const int* stop, FinishArgs* f) {
+    *f = FinishArgs{};
+    f->pb = h->pb;
+    f->inv_n = 1.0 / (double)h->n_s;
+    f->part = (const double*)h->d_pfpart;
+    f->nblk = nblk; f->nimg = L.nimg;
+    f->corr_raw = h->d_corrraw;
+    f->invC = h->d_invC64;
+    f->stop = stop;
+}
+
+// blocks of k_sr_finish: 32 image entries each, then correlators (two per
+// thread up to a slot of partial dots)
+static int finish_grid(const vmc_ctx* h, const FinishArgs& f) {
+    const int nb1 = (f.nimg + 31) / 32;
+    if (f.nimg > h->npf) return nb1;
+    return nb1 + (int)std::max<int64_t>(0, std::min<int64_t>((h->ncp + 511) / 512, kNumPart * kMaxK - nb1));
+}
+
+template <typename AT, int K>
+static int launch_corr(vmc_ctx* h, const AT* T, const int* stop, cudaStream_t st, bool cleared = false);
+
+// pass with FP64 sums over the FP64, FP32 or (gradient only) BF16 store; Obar
+// not null: its product with V goes to part(0), a partial per CTA.  f: what
+// k_sr_finish needs to know of the pass
 static int launch_pass(vmc_ctx* h, const void* s_pf, int store_bytes, int K, bool gather, const double* V, double* T,
-                       const int* stop, cudaStream_t st, int* nblk) {
+                       const double* Obar, const int* stop, cudaStream_t st, FinishArgs* f) {
     vmc_ctx::PassPlan* L;
     int rc = plan_pass(h, K, gather, &L);
     if (rc) return rc;
     const int64_t need = (h->n_s + 3) / 4;   // a few samples per CTA keep small sets spread over the SMs
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(h->nsm, need));
-    if ((size_t)grid * h->npf * K * sizeof(double) > h->pfpart_bytes) return VMC_ERR_UNSUPPORTED;
+    if ((size_t)grid * L->nimg * K * sizeof(double) > h->pfpart_bytes) return VMC_ERR_UNSUPPORTED;
     vmc_ctx::PassRec rec{};
     if (h->prof) {
         rec.a = h->get_event();
@@ -1281,13 +1324,21 @@ static int launch_pass(vmc_ctx* h, const void* s_pf, int store_bytes, int K, boo
     }
     PassArgs a;
     pass_args(h, *L, K, s_pf, V, T, stop, a);
+    a.Obar = Obar;
+    a.obv_part = h->part(0);
     VCK(launch_sr_pass(store_bytes, a, K, gather, grid, L->smem, st));
     h->n_launch++;
     if (h->prof) {
         VCK(cudaEventRecord(rec.b, st));
         h->recs.push_back(rec);
     }
-    *nblk = grid;
+    if (L->nimg == h->npf) {
+        if (K == 1) rc = launch_corr<double, 1>(h, T, stop, st, true);
+        else if (K == 2) rc = launch_corr<double, 2>(h, T, stop, st, true);
+        else rc = launch_corr<double, 4>(h, T, stop, st, true);
+        if (rc) return rc;
+    }
+    finish_args(h, *L, grid, stop, f);
     return VMC_OK;
 }
 
@@ -1377,7 +1428,7 @@ static int launch_stream(vmc_ctx* h, const void* s_pf, const float* V, const flo
     a.V = V; a.invC = invC; a.T = T;
     a.pf_partial = (float*)h->d_pfpart;
     a.stop = stop;
-    a.status = h->d_status;
+    a.status = h->status_word();
     a.spin_limit = h->wait_limit;
     a.buf_bytes = buf;
     kern<<<grid, 32 * nw, smem, st>>>(a);
@@ -1392,9 +1443,9 @@ static int launch_stream(vmc_ctx* h, const void* s_pf, const float* V, const flo
 }
 
 // correlator scatter: one thread-block cluster of kCorrCluster CTAs per
-// correlator, the sums over samples go to d_corrraw
+// correlator, the sums over samples go to d_corrraw (cleared: already zero)
 template <typename AT, int K>
-static int launch_corr(vmc_ctx* h, const AT* T, const int* stop, cudaStream_t st) {
+static int launch_corr(vmc_ctx* h, const AT* T, const int* stop, cudaStream_t st, bool cleared) {
     if (h->ncorr == 0) return VMC_OK;
     size_t smem = (size_t)h->maxd * K * sizeof(AT);
     CorrArgs<AT> a{};
@@ -1405,7 +1456,7 @@ static int launch_corr(vmc_ctx* h, const AT* T, const int* stop, cudaStream_t st
     a.corr_raw = (AT*)h->d_corrraw;
     a.units = h->d_units;
     a.stop = stop;
-    VCK(cudaMemsetAsync(h->d_corrraw, 0, sizeof(AT) * h->ncp * K, st));
+    if (!cleared) VCK(cudaMemsetAsync(h->d_corrraw, 0, sizeof(AT) * h->ncp * K, st));
     if (smem + 1024 > h->smem_optin) {   // histograms beyond shared memory: global additions
         const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>((h->n_s + 255) / 256, 64)),
                         (unsigned)h->ncorr);
@@ -1423,10 +1474,9 @@ static int launch_corr(vmc_ctx* h, const AT* T, const int* stop, cudaStream_t st
     return VMC_OK;
 }
 
-template <typename AT>
 static int reduce_pf(vmc_ctx* h, int nblk, int K, cudaStream_t st) {
     const int n = h->npf * K;
-    k_reduce_pf<AT><<<(n + 31) / 32, 256, 0, st>>>((const AT*)h->d_pfpart, nblk, n, (AT*)h->d_pfraw); h->n_launch++;
+    k_reduce_pf<<<(n + 31) / 32, 256, 0, st>>>((const float*)h->d_pfpart, nblk, n, (float*)h->d_pfraw); h->n_launch++;
     VCK(cudaGetLastError());
     return VMC_OK;
 }
@@ -1435,12 +1485,6 @@ static int reduce_pf(vmc_ctx* h, int nblk, int K, cudaStream_t st) {
 // partial dots per block go to one slot of kNumPart * kMaxK doubles
 static int vgrid(const vmc_ctx* h, int K = 1) {
     int64_t g = (h->nv + 1023) / 1024;
-    return (int)std::max<int64_t>(1, std::min<int64_t>(g, (int64_t)kNumPart * kMaxK / K));
-}
-
-// blocks of the gradient finalize kernel
-static int fin_grid(const vmc_ctx* h, int K = 1) {
-    int64_t g = (h->nv + 255) / 256;
     return (int)std::max<int64_t>(1, std::min<int64_t>(g, (int64_t)kNumPart * kMaxK / K));
 }
 
@@ -1809,77 +1853,91 @@ static int launch_fused(vmc_ctx* h, const float* V, const float* invC, const dou
     return VMC_OK;
 }
 
-// out = (S + shift I) V with K vectors, V/out in AT precision ([K][nv]), over
-// store s_pf whose sample means are Obar of kind `kind`.  obv_part holds
-// vgrid(h, K) partial dots Obar . V unless null (then computed first: the
-// sorted pass centers t_s with it); dot_part receives vgrid(h, K) partial
-// dots out . V.
-template <typename ST, typename AT, int K>
-static int apply_S_impl(vmc_ctx* h, const void* s_pf, int kind, const AT* V, AT* out, double shift,
-                        const int* stop, const double* obv_part, double* dot_part, cudaStream_t st) {
-    const AT* invC;
-    if (sizeof(AT) == 8) invC = (const AT*)h->d_invC64;
-    else invC = (const AT*)h->d_invC32;
-    const double* Obar = h->d_Obar[kind];
-    const AT* ObarA = sizeof(AT) == 8 ? (const AT*)h->d_Obar[kind] : (const AT*)h->d_Obar32[kind];
-    AT* T = (AT*)h->d_T;
-    if (!obv_part) {
-        k_dot_part<double, AT, K><<<vgrid(h, K), 256, 0, st>>>(Obar, V, h->nv, h->part(0), stop); h->n_launch++;
-        VCK(cudaGetLastError());
-        obv_part = h->part(0);
-    }
+// out = (S + shift I) V with K vectors over store s_pf whose sample means are
+// Obar of kind `kind`, FP64 sums.  obv_part holds n_obv partial dots Obar . V;
+// null: the pass forms them in part(0).  dot_part receives partial dots
+// out . V.  nobv, ndot: how many partials of either there are.
+template <typename ST, int K>
+static int apply_S64(vmc_ctx* h, const void* s_pf, int kind, const double* V, double* out, double shift,
+                     const int* stop, const double* obv_part, int n_obv, double* dot_part, cudaStream_t st,
+                     int* nobv = nullptr, int* ndot = nullptr) {
+    FinishArgs f;
+    int rc = launch_pass(h, s_pf, (int)sizeof(ST), K, true, V, (double*)h->d_T, obv_part ? nullptr : h->d_Obar[kind],
+                         stop, st, &f);
+    if (rc) return rc;
+    f.lead_part = obv_part ? obv_part : h->part(0);
+    f.n_lead = obv_part ? n_obv : f.nblk;
+    f.Obar = h->d_Obar[kind];
+    f.V = V;
+    f.shift = shift;
+    f.out = out;
+    f.dot_part = dot_part;
+    const int grid = finish_grid(h, f);
+    VCK(launch_sr_finish(f, K, false, grid, st));
+    h->n_launch++;
+    if (nobv) *nobv = f.n_lead;
+    if (ndot) *ndot = grid;
+    return VMC_OK;
+}
+
+// The same with FP32 sums, V and out in FP32.  obv_part (not null) holds
+// vgrid(h, K) partial dots Obar . V: the sorted pass centers t_s with it;
+// dot_part receives vgrid(h, K) partial dots out . V.  cleared: d_corrraw is
+// zero; out64 (not null) takes the result in FP64 instead of out.
+template <typename ST, int K>
+static int apply_S32(vmc_ctx* h, const void* s_pf, int kind, const float* V, float* out, double shift, const int* stop,
+                     const double* obv_part, double* dot_part, cudaStream_t st, bool cleared = false,
+                     double* out64 = nullptr) {
+    const float* invC = h->d_invC32;
+    float* T = (float*)h->d_T;
     int nblk = 0;
     int rc = VMC_ERR_UNSUPPORTED;
     bool sorted = false;
     const int path = product_path(h, K);
-    if constexpr (sizeof(AT) == 4 && sizeof(ST) == 2 && K == 1) {
+    if constexpr (sizeof(ST) == 2 && K == 1) {
         if (path == VMC_PATH_FUSED) {
-            rc = launch_fused(h, (const float*)V, (const float*)invC, obv_part, (float*)T, stop, st);
+            rc = launch_fused(h, V, invC, obv_part, T, stop, st, nullptr, cleared);
             if (rc != VMC_OK && rc != VMC_ERR_UNSUPPORTED) return rc;
             sorted = rc == VMC_OK;
         }
     }
-    if constexpr (sizeof(AT) == 4 && sizeof(ST) == 2) {
+    if constexpr (sizeof(ST) == 2) {
         if (!sorted && (path == VMC_PATH_SORTED || path == VMC_PATH_FUSED || path == VMC_PATH_COMPACT) &&
             h->use_sorted && h->d_G) {
-            rc = launch_sorted<K>(h, (const float*)V, (const float*)invC, obv_part, (float*)T, stop, st);
+            rc = launch_sorted<K>(h, V, invC, obv_part, T, stop, st, nullptr, cleared);
             if (rc != VMC_OK && rc != VMC_ERR_UNSUPPORTED) return rc;
             sorted = rc == VMC_OK;
         }
     }
-    if constexpr (sizeof(AT) == 4 && K <= 2) {
+    if constexpr (K <= 2) {
         if (rc == VMC_ERR_UNSUPPORTED && path != VMC_PATH_GENERIC && h->use_stream)
-            rc = launch_stream<ST, K>(h, s_pf, (const float*)V, (const float*)invC, (float*)T, stop, st, &nblk);
+            rc = launch_stream<ST, K>(h, s_pf, V, invC, T, stop, st, &nblk);
     }
-    if (rc == VMC_ERR_UNSUPPORTED) {
-        if constexpr (sizeof(AT) == 8) rc = launch_pass(h, s_pf, (int)sizeof(ST), K, true, V, T, stop, st, &nblk);
-        else rc = launch_main<ST, K>(h, s_pf, V, invC, T, stop, st, &nblk);
-    }
+    if (rc == VMC_ERR_UNSUPPORTED) rc = launch_main<ST, K>(h, s_pf, V, invC, T, stop, st, &nblk);
     if (rc) return rc;
     if (!sorted) {   // the sorted pass scatters the correlators itself
-        rc = launch_corr<AT, K>(h, T, stop, st);
+        rc = launch_corr<float, K>(h, T, stop, st, cleared);
         if (rc) return rc;
-        rc = reduce_pf<AT>(h, nblk, K, st);
+        rc = reduce_pf(h, nblk, K, st);
         if (rc) return rc;
     }
-    FinArgs<AT, AT> f{};
+    FinArgs f{};
     f.pb = h->pb;
-    f.n_s = h->n_s;
     f.inv_n = 1.0 / (double)h->n_s;
     f.centered = sorted ? 1 : 0;
-    f.pf_partial = (const AT*)h->d_pfpart;
-    f.pf_raw = (const AT*)h->d_pfraw;
-    f.corr_raw = (const AT*)h->d_corrraw;
+    f.pf_raw = (const float*)h->d_pfraw;
+    f.corr_raw = (const float*)h->d_corrraw;
     f.invC = invC;
-    f.ObarA = ObarA;
+    f.Obar = h->d_Obar32[kind];
     f.obv_part = obv_part;
     f.n_obv_part = vgrid(h, K);
     f.V = V;
     f.shift = shift;
     f.out = out;
+    f.out64 = out64;
     f.dot_part = dot_part;
     f.stop = stop;
-    k_finalize_S<AT, AT, K><<<vgrid(h, K), 256, 0, st>>>(f); h->n_launch++;
+    k_finalize_S<K><<<vgrid(h, K), 256, 0, st>>>(f); h->n_launch++;
     VCK(cudaGetLastError());
     return VMC_OK;
 }
@@ -1906,28 +1964,16 @@ static int gradient_pass(vmc_ctx* h, int kind, double* g, cudaStream_t st) {
     double* T = (double*)h->d_T;
     k_build_T_grad<<<kNumPart, 256, 0, st>>>(h->d_E, h->n_s, T, h->part(1)); h->n_launch++;
     VCK(cudaGetLastError());
-    int nblk = 0, rc;
-    rc = launch_pass(h, src, kind == 0 ? 8 : kind == 1 ? 4 : 2, 2, false, nullptr, T, nullptr, st, &nblk);
+    FinishArgs f;
+    int rc = launch_pass(h, src, kind == 0 ? 8 : kind == 1 ? 4 : 2, 2, false, nullptr, T, nullptr, nullptr, st, &f);
     if (rc) return rc;
-    rc = launch_corr<double, 2>(h, T, nullptr, st);
-    if (rc) return rc;
-    rc = reduce_pf<double>(h, nblk, 2, st);
-    if (rc) return rc;
-    FinArgs<double, double> f{};
-    f.pb = h->pb;
-    f.n_s = h->n_s;
-    f.inv_n = 1.0 / (double)h->n_s;
-    f.pf_partial = (const double*)h->d_pfpart;
-    f.pf_raw = h->d_pfraw;
-    f.corr_raw = h->d_corrraw;
-    f.invC = h->d_invC64;
+    f.lead_part = h->part(1);
+    f.n_lead = kNumPart;
     f.Obar_out = h->d_Obar[kind];
+    f.Obar32_out = h->d_Obar32[kind];
     f.g_out = g;
-    f.E_sum = h->part(1);
-    f.n_E_part = kNumPart;
-    k_finalize_grad<double><<<fin_grid(h), 256, 0, st>>>(f); h->n_launch++;
-    k_cast<float><<<kNumPart, 256, 0, st>>>(h->d_Obar[kind], h->d_Obar32[kind], h->nv, 1.0); h->n_launch++;
-    VCK(cudaGetLastError());
+    VCK(launch_sr_finish(f, 2, true, finish_grid(h, f), st));
+    h->n_launch++;
     h->obar_ok[kind] = true;
     return VMC_OK;
 }
@@ -1982,7 +2028,7 @@ extern "C" int sr_gradient(vmc_handle h, double* g, double* e_stats, int store, 
 }
 
 static size_t main_smem(const vmc_ctx* h, int K, size_t at_bytes) {
-    if (at_bytes == 8) return pass_smem(h->npf, h->P, K, true, 1);
+    if (at_bytes == 8) return pass_smem(h->npf, h->npf, h->P, K, true, 1);
     return (size_t)h->npf * K * at_bytes * 2 + (size_t)h->M * 4 + 16 * 64;
 }
 
@@ -2009,27 +2055,22 @@ static int apply_S_dispatch(vmc_ctx* h, const double* V, double* out, double shi
     if (rc0) return rc0;
     switch (store) {
         case VMC_STORE_FP64:
-            return apply_S_impl<double, double, K>(h, h->d_pf64, kind, V, out, shift, nullptr, nullptr, nullptr, st);
+            return apply_S64<double, K>(h, h->d_pf64, kind, V, out, shift, nullptr, nullptr, 0, nullptr, st);
         case VMC_STORE_FP32:
-            return apply_S_impl<float, double, K>(h, h->d_pf32, kind, V, out, shift, nullptr, nullptr, nullptr, st);
+            return apply_S64<float, K>(h, h->d_pf32, kind, V, out, shift, nullptr, nullptr, 0, nullptr, st);
         case VMC_STORE_BF16:
         case VMC_STORE_FP32_F32ACC: {
             const void* src = store == VMC_STORE_BF16 ? (const void*)h->d_pf16 : (const void*)h->d_pf32;
             if (!src) return VMC_ERR_STATE;
-            const int64_t n = h->nv * K;
-            k_cast<float><<<kNumPart, 256, 0, st>>>(V, h->d_b32, n, 1.0); h->n_launch++;
+            k_cast_dot<K><<<vgrid(h, K), 256, 0, st>>>(V, h->d_b32, h->d_Obar[kind], h->nv, h->part(0),
+                                                       (float*)h->d_corrraw, h->ncp * K);
+            h->n_launch++;
             VCK(cudaGetLastError());
-            int rc = store == VMC_STORE_BF16
-                         ? apply_S_impl<__nv_bfloat16, float, K>(h, src, kind, h->d_b32, h->d_q32, shift, nullptr,
-                                                                 nullptr, nullptr, st)
-                         : apply_S_impl<float, float, K>(h, src, kind, h->d_b32, h->d_q32, shift, nullptr, nullptr,
-                                                         nullptr, st);
-            if (rc) return rc;
-            // widen back to FP64
-            VCK(cudaMemsetAsync(out, 0, sizeof(double) * n, st));
-            k_axpy_to64<float><<<kNumPart, 256, 0, st>>>(out, h->d_q32, 1.0, n); h->n_launch++;
-            VCK(cudaGetLastError());
-            return VMC_OK;
+            return store == VMC_STORE_BF16
+                       ? apply_S32<__nv_bfloat16, K>(h, src, kind, h->d_b32, nullptr, shift, nullptr, h->part(0), nullptr,
+                                                     st, true, out)
+                       : apply_S32<float, K>(h, src, kind, h->d_b32, nullptr, shift, nullptr, h->part(0), nullptr, st,
+                                             true, out);
         }
         default:
             return VMC_ERR_INVALID_ARG;
@@ -2079,13 +2120,12 @@ static int time_path(vmc_ctx* h, int path, int reps, cudaStream_t st, double* ms
     const int64_t n = h->nv * K;
     // a zero vector: the passes do the same work for any input
     if (cudaMemsetAsync(h->d_b32, 0, sizeof(float) * n, st) != cudaSuccess) return VMC_ERR_CUDA;
-    int rc = apply_S_impl<__nv_bfloat16, float, K>(h, h->d_pf16, 2, h->d_b32, h->d_q32, 1e-3, nullptr, nullptr,
-                                                  nullptr, st);   // warm-up (builds the path's copies)
+    if (cudaMemsetAsync(h->part(0), 0, sizeof(double) * vgrid(h, K) * K, st) != cudaSuccess) return VMC_ERR_CUDA;   // Obar . V
+    int rc = apply_S32<__nv_bfloat16, K>(h, h->d_pf16, 2, h->d_b32, h->d_q32, 1e-3, nullptr, h->part(0), nullptr, st);   // warm-up (builds the path's copies)
     cudaEvent_t e0 = h->get_event(), e1 = h->get_event();
     if (!rc) rc = cudaEventRecord(e0, st) == cudaSuccess ? VMC_OK : VMC_ERR_CUDA;
     for (int r = 0; r < reps && !rc; ++r)
-        rc = apply_S_impl<__nv_bfloat16, float, K>(h, h->d_pf16, 2, h->d_b32, h->d_q32, 1e-3, nullptr, nullptr,
-                                                  nullptr, st);
+        rc = apply_S32<__nv_bfloat16, K>(h, h->d_pf16, 2, h->d_b32, h->d_q32, 1e-3, nullptr, h->part(0), nullptr, st);
     if (!rc) rc = cudaEventRecord(e1, st) == cudaSuccess ? VMC_OK : VMC_ERR_CUDA;
     float t = 0.f;
     if (!rc) rc = cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&t, e0, e1) == cudaSuccess
@@ -2219,9 +2259,12 @@ static int cg_loop(vmc_ctx* h, const void* s_pf, int kind, const VT* b, VT* x, V
                     k_cg_fxr<float><<<vg, 256, 0, st>>>(f); h->n_launch++;
                 }
             } else {
-                int rc = apply_S_impl<ST, VT, 1>(h, s_pf, kind, p, q, shift, h->d_stop, obp_part, pAp_part, st);
+                int rc, ndot = vg;
+                if constexpr (sizeof(VT) == 8)
+                    rc = apply_S64<ST, 1>(h, s_pf, kind, p, q, shift, h->d_stop, obp_part, vg, pAp_part, st, nullptr, &ndot);
+                else rc = apply_S32<ST, 1>(h, s_pf, kind, p, q, shift, h->d_stop, obp_part, pAp_part, st);
                 if (rc) return rc;
-                k_cg_xr<VT><<<vg, 256, 0, st>>>(x, r, p, q, n, pAp_part, vg, h->d_scal, rr_part, h->d_stop); h->n_launch++;
+                k_cg_xr<VT><<<vg, 256, 0, st>>>(x, r, p, q, n, pAp_part, ndot, h->d_scal, rr_part, h->d_stop); h->n_launch++;
             }
             k_cg_p<VT><<<vg, 256, 0, st>>>(r, p, n, rr_part, vg, h->d_scal, ObarV, obp_part, pp_part,
                                            h->d_stop, max_iter); h->n_launch++;
@@ -2250,7 +2293,7 @@ static int cg_loop(vmc_ctx* h, const void* s_pf, int kind, const VT* b, VT* x, V
 template <typename ST>
 static int residual64(vmc_ctx* h, const void* s_pf, int kind, const double* g, const double* x, double* y,
                       double shift, double* rr, cudaStream_t st) {
-    int rc = apply_S_impl<ST, double, 1>(h, s_pf, kind, x, h->d_t64, shift, nullptr, nullptr, nullptr, st);
+    int rc = apply_S64<ST, 1>(h, s_pf, kind, x, h->d_t64, shift, nullptr, nullptr, 0, nullptr, st);
     if (rc) return rc;
     k_sub<<<kNumPart, 256, 0, st>>>(g, h->d_t64, y, h->nv, h->part(6)); h->n_launch++;
     VCK(cudaGetLastError());
@@ -2354,7 +2397,7 @@ static int inner_block(vmc_ctx* h, const double* r, double rnorm, double* z, dou
     max_iter = std::min(max_iter, kBlockInnerMax);
     for (int done = 0; !done;) {
         for (int j = 0; j < kChunk; ++j) {
-            int rc = apply_S_impl<__nv_bfloat16, float, 4>(h, h->d_pf16, 2, P, Q, shift, h->d_stop, obp_part, nullptr, st);
+            int rc = apply_S32<__nv_bfloat16, 4>(h, h->d_pf16, 2, P, Q, shift, h->d_stop, obp_part, nullptr, st);
             if (rc) return rc;
             k_bcg_gram<<<vg, 256, 0, st>>>(P, Q, n, gpart, h->d_stop);
             k_bcg_alpha<<<1, 256, 0, st>>>(gpart, vg, S, h->d_stop);
@@ -2420,8 +2463,8 @@ static int fcg_mixed(vmc_ctx* h, const double* g, double shift, double tol, int 
     // FP64 accumulation
     const bool outer64 = mode == VMC_CG_MIXED64;
     for (int outer = 0; outer < 200; ++outer) {
-        rc = outer64 ? apply_S_impl<double, double, 1>(h, h->d_pf64, 0, p, q, shift, nullptr, nullptr, nullptr, st)
-                     : apply_S_impl<float, double, 1>(h, h->d_pf32, 1, p, q, shift, nullptr, nullptr, nullptr, st);
+        rc = outer64 ? apply_S64<double, 1>(h, h->d_pf64, 0, p, q, shift, nullptr, nullptr, 0, nullptr, st)
+                     : apply_S64<float, 1>(h, h->d_pf32, 1, p, q, shift, nullptr, nullptr, 0, nullptr, st);
         if (rc) return rc;
         inf->residual_products++;
         double pq = dot64(h, p, q, st, &rc);
@@ -2530,7 +2573,7 @@ extern "C" int sr_update(vmc_handle h, const double* y, double tau, int store, d
     a.e_part = h->part(0); a.ne = kNumPart;
     a.oy_part = h->part(1); a.noy = kNumPart;
     a.x0 = h->d_scal + kScalX0;
-    a.status = h->d_status;
+    a.status = h->status_word();
     k_sr_update<<<vgrid(h, 1), 256, 0, st>>>(a); h->n_launch++;
     VCK(cudaGetLastError());
     // the stored samples belong to the old parameters
@@ -2578,10 +2621,12 @@ extern "C" int sr_local_product(vmc_handle h, const double* v, double* out, int 
     cudaStream_t st = (cudaStream_t)stream;
     // out = S v with shift 0 (uncentered pass, covariance term in the finalize),
     // then back to the plain sum; Obar . v is left in part(0) by the product
-    int rc = kind == 0 ? apply_S_impl<double, double, 1>(h, h->d_pf64, kind, v, out, 0.0, nullptr, nullptr, nullptr, st)
-                       : apply_S_impl<float, double, 1>(h, h->d_pf32, kind, v, out, 0.0, nullptr, nullptr, nullptr, st);
+    int nobv = 0;
+    int rc = kind == 0
+                 ? apply_S64<double, 1>(h, h->d_pf64, kind, v, out, 0.0, nullptr, nullptr, 0, nullptr, st, &nobv)
+                 : apply_S64<float, 1>(h, h->d_pf32, kind, v, out, 0.0, nullptr, nullptr, 0, nullptr, st, &nobv);
     if (rc) return rc;
-    k_uncenter<<<kNumPart, 256, 0, st>>>(out, h->d_Obar[kind], h->part(0), vgrid(h, 1), (double)h->n_s, h->nv);
+    k_uncenter<<<kNumPart, 256, 0, st>>>(out, h->d_Obar[kind], h->part(0), nobv, (double)h->n_s, h->nv);
     h->n_launch++;
     VCK(cudaGetLastError());
     return VMC_OK;
@@ -3009,7 +3054,7 @@ extern "C" int lm_update(vmc_handle h, const double* x, double Sx0, void* stream
     a.C64 = h->d_C64; a.C32 = h->d_C32; a.invC64 = h->d_invC64; a.invC32 = h->d_invC32;
     a.F64 = h->d_F64; a.F32 = h->d_F32; a.pq_of = h->d_pq_of;
     a.ncp = h->ncp; a.npf = h->npf; a.M = h->M;
-    a.status = h->d_status;
+    a.status = h->status_word();
     k_lm_update<<<vgrid(h, 1), 256, 0, st>>>(a, x, 1.0 / Sx0); h->n_launch++;
     VCK(cudaGetLastError());
     h->obar_ok[0] = h->obar_ok[1] = h->obar_ok[2] = false;
@@ -3084,17 +3129,17 @@ extern "C" int sr_apply_S_batch(const vmc_handle* hs, int n, const double* const
         vmc_ctx* h = hs[b];
         int rc = ensure_obar(h, kind, st);
         if (rc) return rc;
-        k_dot_part<double, double, 1><<<vgrid(h, 1), 256, 0, st>>>(h->d_Obar[kind], V[b], h->nv, h->part(0), nullptr);
-        h->n_launch++;
         vmc_ctx::PassPlan* L;
         if ((rc = plan_pass(h, 1, true, &L))) return rc;
         smem = std::max(smem, L->smem);
         const double share = (double)h->n_s * (h->P + h->ncorr) / work;
         int g = (int)std::ceil(share * 2 * h0->nsm);
         g = (int)std::max<int64_t>(1, std::min<int64_t>(g, (h->n_s + 15) / 16));
-        g = std::min<int64_t>(g, (int64_t)(h->pfpart_bytes / ((size_t)h->npf * sizeof(double))));
+        g = std::min<int64_t>(g, (int64_t)(h->pfpart_bytes / ((size_t)L->nimg * sizeof(double))));
         cta0[b + 1] = cta0[b] + g;
         pass_args(h, *L, 1, store_ptr(h, kind), V[b], (double*)h->d_T, nullptr, args[b]);
+        args[b].Obar = h->d_Obar[kind];
+        args[b].obv_part = h->part(0);
     }
     void* dbuf = nullptr;
     const size_t abytes = round_up(sizeof(PassArgs) * n, 256);
@@ -3108,27 +3153,19 @@ extern "C" int sr_apply_S_batch(const vmc_handle* hs, int n, const double* const
     h0->n_launch++;
     for (int b = 0; b < n; ++b) {
         vmc_ctx* h = hs[b];
-        if ((rc = launch_corr<double, 1>(h, (double*)h->d_T, nullptr, st))) return rc;
-        if ((rc = reduce_pf<double>(h, cta0[b + 1] - cta0[b], 1, st))) return rc;
-        FinArgs<double, double> f{};
-        f.pb = h->pb;
-        f.n_s = h->n_s;
-        f.inv_n = 1.0 / (double)h->n_s;
-        f.centered = 0;
-        f.pf_partial = (const double*)h->d_pfpart;
-        f.pf_raw = h->d_pfraw;
-        f.corr_raw = h->d_corrraw;
-        f.invC = h->d_invC64;
-        f.ObarA = h->d_Obar[kind];
-        f.obv_part = h->part(0);
-        f.n_obv_part = vgrid(h, 1);
+        vmc_ctx::PassPlan* L;
+        if ((rc = plan_pass(h, 1, true, &L))) return rc;
+        if (L->nimg == h->npf && (rc = launch_corr<double, 1>(h, (double*)h->d_T, nullptr, st, true))) return rc;
+        FinishArgs f;
+        finish_args(h, *L, cta0[b + 1] - cta0[b], nullptr, &f);
+        f.lead_part = h->part(0);
+        f.n_lead = f.nblk;
+        f.Obar = h->d_Obar[kind];
         f.V = V[b];
         f.shift = shift;
         f.out = out[b];
-        f.dot_part = nullptr;
-        f.stop = nullptr;
-        k_finalize_S<double, double, 1><<<vgrid(h, 1), 256, 0, st>>>(f); h->n_launch++;
-        VCK(cudaGetLastError());
+        VCK(launch_sr_finish(f, 1, false, finish_grid(h, f), st));
+        h->n_launch++;
     }
     // the host copies of the argument blocks must outlive the launch's copies
     VCK(cudaStreamSynchronize(st));

@@ -151,12 +151,37 @@ struct PassArgs {
     const double* V;          // [K][nv]
     const double* invC;       // [ncp]
     double* T;                // [n_s][K]
-    double* pf_partial;       // [gridDim][npf][K]
+    double* pf_partial;       // [gridDim][nimg][K]
+    int nimg;                 // entries of an image: npf, or npf + ncp with the correlators (no shared blocks)
+    const double* Obar;       // not null: obv_part[gridDim][K] = partial Obar . V
+    double* obv_part;
+    double* clear;            // not null: [ncp][K] to be cleared
     int ni;                   // images; pass_warps(K) / ni warps share one
     int bounds[pass_warps(1) + 1];   // first orbital p of each of an image's owners, then M
     const int* stop;
 };
-size_t pass_smem(int npf, int P, int K, bool gather, int ni);
+// what follows the pass (k_sr_finish)
+struct FinishArgs {
+    DevProblem pb;
+    double inv_n;             // 1 / n_s
+    const double* part;       // [nblk][nimg][K] the pass's images
+    int nblk, nimg;
+    const double* corr_raw;   // [ncp][K] correlator sums (nimg = npf)
+    const double* invC;
+    const double* lead_part;  // partials of Obar . V, or of the sum of E_L (gradient)
+    int n_lead;
+    const double* Obar;       // product
+    const double* V;
+    double shift;
+    double* out;
+    double* dot_part;         // [gridDim][K] partial out . V (may be null)
+    double* Obar_out;         // gradient
+    float* Obar32_out;
+    double* g_out;
+    const int* stop;
+};
+cudaError_t launch_sr_finish(const FinishArgs& a, int K, bool grad, int grid, cudaStream_t st);
+size_t pass_smem(int npf, int nimg, int P, int K, bool gather, int ni);
 cudaError_t launch_sr_pass(int store_bytes, const PassArgs& a, int K, bool gather, int grid, size_t smem, cudaStream_t st);
 cudaError_t launch_sr_pass_batch(int store_bytes, int blocks, size_t smem, cudaStream_t st, const PassArgs* args,
                                  const int* cta0, int n);
@@ -175,43 +200,38 @@ struct CorrArgs {
 
 constexpr int kCorrCluster = 8;  // CTAs per correlator (one thread-block cluster)
 
-template <typename AT, typename VT>
+// out = raw / n - Obar (Obar . V) + shift V of the passes with FP32 sums
 struct FinArgs {
     DevProblem pb;
-    int64_t n_s;
     double inv_n;           // 1 / n_s
     int centered;           // the pass scattered t_s - Obar . V: skip the Obar term
-    const AT* pf_partial;
-    const AT* pf_raw;       // [npf][K] pairing-block sums
-    const AT* corr_raw;     // [ncp][K] correlator sums
-    const AT* ObarA;        // [nv] Obar in AT (S mode, uncentered)
-    const AT* invC;
-    const double* obv_part; // [nblk][K] partial dots Obar . V (S mode, uncentered)
+    const float* pf_raw;    // [npf][K] pairing-block sums
+    const float* corr_raw;  // [ncp][K] correlator sums
+    const float* Obar;      // [nv] (uncentered)
+    const float* invC;
+    const double* obv_part; // [nblk][K] partial dots Obar . V (uncentered)
     int n_obv_part;
-    const VT* V;            // [K][nv]
+    const float* V;         // [K][nv]
     double shift;
-    VT* out;                // [K][nv]
+    float* out;             // [K][nv], or
+    double* out64;          // not null: the same values in FP64 instead
     double* dot_part;       // [gridDim][K] partial out . V (may be null)
-    // gradient mode
-    double* Obar_out;
-    double* g_out;
-    const double* E_sum;    // [nblk] partial sums of E (gradient mode)
-    int n_E_part;
     const int* stop;
 };
-
 
 template <typename ST, int K> __global__ void __launch_bounds__(512) k_sr_main(MainArgs<float> a);
 template <typename AT, int K>
 __global__ void __cluster_dims__(kCorrCluster, 1, 1) __launch_bounds__(256) k_corr_scatter(CorrArgs<AT> a);
 template <typename AT, int K> __global__ void __launch_bounds__(256) k_corr_scatter_global(CorrArgs<AT> a);
-template <typename AT, typename VT, int K> __global__ void __launch_bounds__(256) k_finalize_S(FinArgs<AT, VT> a);
-template <typename AT> __global__ void __launch_bounds__(256) k_finalize_grad(FinArgs<AT, double> a);
+template <int K> __global__ void __launch_bounds__(256) k_finalize_S(FinArgs a);
+// dst = (float)src [K][nv], partial dots Obar . dst, and clear[i] = 0 for i < nclear
+template <int K>
+__global__ void __launch_bounds__(256) k_cast_dot(const double* src, float* dst, const double* Obar, int64_t n, double* part,
+                                                  float* clear, int64_t nclear);
 __global__ void k_build_T_grad(const double* E, int64_t n_s, double* T, double* E_part);
 template <typename TA, typename TB, int K>
 __global__ void __launch_bounds__(256) k_dot_part(const TA* x, const TB* y, int64_t n, double* part, const int* stop);
-template <typename AT>
-__global__ void __launch_bounds__(256) k_reduce_pf(const AT* part, int nblk, int npfK, AT* raw);
+__global__ void __launch_bounds__(256) k_reduce_pf(const float* part, int nblk, int npfK, float* raw);
 __global__ void k_transpose_cidx(const cstate_t* cidx, int ncst, int ncorr, int64_t n_s, cstate_t* cidxT);
 template <typename VT> __global__ void k_cast(const double* src, VT* dst, int64_t n, double scale);
 

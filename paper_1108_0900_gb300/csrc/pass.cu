@@ -101,22 +101,47 @@ __device__ void pass_run(const PassArgs& a, int cta, int ncta, unsigned char* sm
     using A = typename std::conditional<std::is_same<ST, float>::value, PairAcc, PlainAcc>::type;
     using E = typename A::Elem;
     const DevProblem& pb = a.pb;
-    const int npf = pb.npf, N = pb.N, P = pb.P, ni = a.ni, owners = NW / ni;
-    E* img = (E*)smem;                                           // [ni][npf][K]
-    E* vpf = img + (size_t)ni * npf * K;                         // [npf][K]
+    const int npf = pb.npf, N = pb.N, P = pb.P, ni = a.ni, owners = NW / ni, nimg = a.nimg;
+    E* img = (E*)smem;                                           // [ni][nimg][K]
+    E* vpf = img + (size_t)ni * nimg * K;                        // [npf][K]
     TileBuf<E, K, NW>* buf = (TileBuf<E, K, NW>*)(vpf + (GATHER ? (size_t)npf * K : 0));   // [2]
     uint32_t* ft = (uint32_t*)(buf + 2);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < ni * npf * K; i += blockDim.x) img[i] = A::make(0.0);
+    for (int i = threadIdx.x; i < ni * nimg * K; i += blockDim.x) img[i] = E{};
     if (GATHER)
         for (int i = threadIdx.x; i < npf; i += blockDim.x)
 #pragma unroll
             for (int kk = 0; kk < K; ++kk) vpf[i * K + kk] = A::make(a.V[kk * pb.nv + pb.ncp + i]);
     for (int i = threadIdx.x; i < P; i += blockDim.x) ft[i] = a.fulltab[i];
+    // on the side: this CTA's share of Obar . V and of clearing the correlator sums
+    if (GATHER && a.Obar) {
+        double* red = (double*)buf;   // [K][NW]
+        const int64_t per = (pb.nv + ncta - 1) / ncta, i1 = min(pb.nv, (cta + 1) * per);
+        double d[K] = {};
+        for (int64_t i = cta * per + threadIdx.x; i < i1; i += blockDim.x) {
+            const double o = a.Obar[i];
+#pragma unroll
+            for (int kk = 0; kk < K; ++kk) d[kk] += o * a.V[kk * pb.nv + i];
+        }
+#pragma unroll
+        for (int kk = 0; kk < K; ++kk) {
+            d[kk] = warp_sum(d[kk]);
+            if (lane == 0) red[kk * NW + wid] = d[kk];
+        }
+        __syncthreads();
+        if (threadIdx.x < K) {
+            double x = 0.0;
+            for (int w = 0; w < NW; ++w) x += red[threadIdx.x * NW + w];
+            a.obv_part[cta * K + threadIdx.x] = x;
+        }
+    }
+    if (a.clear)
+        for (int64_t i = (int64_t)cta * blockDim.x + threadIdx.x; i < pb.ncp * K; i += (int64_t)ncta * blockDim.x)
+            a.clear[i] = 0.0;
     __syncthreads();
     const ST* pf = (const ST*)a.s_pf;
     const int im = wid / owners, own = wid % owners;
-    E* my = img + (size_t)im * npf * K;
+    E* my = img + (size_t)im * nimg * K;
     const int64_t per = (a.n_s + ncta - 1) / ncta;
     const int64_t s0 = min(a.n_s, cta * per), s1 = min(a.n_s, s0 + per);
     int cur = 0;
@@ -216,15 +241,121 @@ __device__ void pass_run(const PassArgs& a, int cta, int ncta, unsigned char* sm
                             my[pq[u] * K + kk] = x[u][kk];
                         }
             }
+            if (nimg > npf)   // the correlators' part in FP64 (1 / C enters at the end): a block each, so no two meet
+                for (int c = own * 32 + lane; c < pb.ncorr; c += 32 * owners) {
+                    double* y = (double*)(my + (npf + pb.corr_off[c] + a.s_cidx[(sb + j) * a.ncst + c]) * K);
+#pragma unroll
+                    for (int kk = 0; kk < K; ++kk) y[kk] += a.T[(sb + j) * K + kk];
+                }
             __syncwarp();   // the next sample's elements may meet these addresses in other lanes
         }
     }
     __syncthreads();
-    double* dst = a.pf_partial + (size_t)cta * npf * K;
+    double* dst = a.pf_partial + (size_t)cta * nimg * K;
     for (int i = threadIdx.x; i < npf * K; i += blockDim.x) {
         E x = img[i];
-        for (int k = 1; k < ni; ++k) A::sum(x, img[(size_t)k * npf * K + i]);
+        for (int k = 1; k < ni; ++k) A::sum(x, img[(size_t)k * nimg * K + i]);
         dst[i] = A::value(x);
+    }
+    for (int i = npf * K + threadIdx.x; i < nimg * K; i += blockDim.x) {
+        double x = 0.0;
+        for (int k = 0; k < ni; ++k) x += ((double*)img)[(size_t)k * nimg * K + i];
+        dst[i] = x;
+    }
+}
+
+// The CTAs' images added up, and what follows: out = raw / n - Obar (Obar . V)
+// + shift V with partial out . V, or (GRAD) the means and the gradient.  Blocks
+// [0, ceil(nimg / 32)) take 32 image entries each, 8 slices of the images; the
+// other blocks the correlator sums that another kernel left in corr_raw.
+// A small product is its launches: with Obar . V, the clearing and the correlators
+// in the pass and everything after it here, 4x4 lattice, 4,096 samples, one vector
+// went from five kernels and a memset at 75 us a call to two at 47.
+template <int K, bool GRAD>
+__global__ void __launch_bounds__(256) k_sr_finish(FinishArgs a) {
+    if (a.stop && *a.stop) return;
+    __shared__ double red[8][K][33];
+    __shared__ double lead[K];   // Obar . V, or <E_L>
+    const DevProblem& pb = a.pb;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (w == 0) {
+#pragma unroll
+        for (int kk = 0; kk < (GRAD ? 1 : K); ++kk) {
+            const double x = warp_sum_partials(a.lead_part, a.n_lead, kk, GRAD ? 1 : K);
+            if (lane == 0) lead[kk] = GRAD ? x * a.inv_n : x;
+        }
+    }
+    const int nb1 = (a.nimg + 31) / 32;
+    double dot[K] = {};
+    auto finish = [&](int64_t k, double* raw) {   // parameter k, its sums
+#pragma unroll
+        for (int kk = 0; kk < K; ++kk) raw[kk] = (k < pb.ncp ? raw[kk] * a.invC[k] : raw[kk]) * a.inv_n;
+        if (GRAD) {
+            a.Obar_out[k] = raw[0];
+            a.Obar32_out[k] = (float)raw[0];
+            a.g_out[k] = raw[1] - lead[0] * raw[0];
+        } else {
+            const double ob = a.Obar[k];
+#pragma unroll
+            for (int kk = 0; kk < K; ++kk) {
+                const double v = a.V[kk * pb.nv + k], o = raw[kk] - ob * lead[kk] + a.shift * v;
+                a.out[kk * pb.nv + k] = o;
+                dot[kk] += o * v;
+            }
+        }
+    };
+    if ((int)blockIdx.x < nb1) {
+        const int i = blockIdx.x * 32 + lane;
+        double s[K] = {};
+        if (i < a.nimg)
+            for (int b0 = w; b0 < a.nblk; b0 += 64) {   // eight images in flight per thread
+                double x[8][K];
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+#pragma unroll
+                    for (int kk = 0; kk < K; ++kk)
+                        x[u][kk] = b0 + 8 * u < a.nblk ? a.part[((int64_t)(b0 + 8 * u) * a.nimg + i) * K + kk] : 0.0;
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+#pragma unroll
+                    for (int kk = 0; kk < K; ++kk) s[kk] += x[u][kk];
+            }
+#pragma unroll
+        for (int kk = 0; kk < K; ++kk) red[w][kk][lane] = s[kk];
+        __syncthreads();
+        if (w == 0 && i < a.nimg) {
+            double raw[K];
+#pragma unroll
+            for (int kk = 0; kk < K; ++kk) {
+                raw[kk] = 0.0;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) raw[kk] += red[j][kk][lane];
+            }
+            finish(i < pb.npf ? pb.ncp + i : i - pb.npf, raw);
+        }
+    } else {
+        __syncthreads();
+        const int64_t stride = (int64_t)(gridDim.x - nb1) * blockDim.x;
+        for (int64_t k = (int64_t)(blockIdx.x - nb1) * blockDim.x + threadIdx.x; k < pb.ncp; k += stride) {
+            double raw[K];
+#pragma unroll
+            for (int kk = 0; kk < K; ++kk) raw[kk] = a.corr_raw[k * K + kk];
+            finish(k, raw);
+        }
+    }
+    if (!GRAD && a.dot_part) {
+        __syncthreads();
+#pragma unroll
+        for (int kk = 0; kk < K; ++kk) {
+            const double x = warp_sum(dot[kk]);
+            if (lane == 0) red[w][kk][0] = x;
+        }
+        __syncthreads();
+        if (threadIdx.x < K) {
+            double x = 0.0;
+            for (int j = 0; j < 8; ++j) x += red[j][threadIdx.x][0];
+            a.dot_part[blockIdx.x * K + threadIdx.x] = x;
+        }
     }
 }
 
@@ -266,11 +397,11 @@ cudaError_t launch_k(const PassArgs& a, int K, bool gather, int grid, size_t sme
 }  // namespace
 
 // shared memory with ni images (a table or image entry is 8 bytes in either arithmetic)
-size_t pass_smem(int npf, int P, int K, bool gather, int ni) {
+size_t pass_smem(int npf, int nimg, int P, int K, bool gather, int ni) {
     const size_t tile = K == 1   ? sizeof(TileBuf<double, 1, pass_warps(1)>)
                         : K == 2 ? sizeof(TileBuf<double, 2, pass_warps(2)>)
                                  : sizeof(TileBuf<double, 4, pass_warps(4)>);
-    return (size_t)npf * K * 8 * (ni + (gather ? 1 : 0)) + 2 * tile + (size_t)P * 4;
+    return ((size_t)nimg * ni + (gather ? npf : 0)) * K * 8 + 2 * tile + (size_t)P * 4;
 }
 
 cudaError_t launch_sr_pass(int store_bytes, const PassArgs& a, int K, bool gather, int grid, size_t smem, cudaStream_t st) {
@@ -285,6 +416,14 @@ cudaError_t launch_sr_pass_batch(int store_bytes, int blocks, size_t smem, cudaS
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<blocks, 32 * pass_warps(1), smem, st>>>(args, cta0, n);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sr_finish(const FinishArgs& a, int K, bool grad, int grid, cudaStream_t st) {
+    if (grad) k_sr_finish<2, true><<<grid, 256, 0, st>>>(a);
+    else if (K == 1) k_sr_finish<1, false><<<grid, 256, 0, st>>>(a);
+    else if (K == 2) k_sr_finish<2, false><<<grid, 256, 0, st>>>(a);
+    else k_sr_finish<4, false><<<grid, 256, 0, st>>>(a);
     return cudaGetLastError();
 }
 

@@ -138,8 +138,7 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[K], double* out) 
 
 // Reduce the per-CTA pairing-block images: raw[pq][kk] = sum_b part[b][pq][kk].
 // Block = 32 parameter slots x 8 CTA slices; a warp covers one slice.
-template <typename AT>
-__global__ void __launch_bounds__(256) k_reduce_pf(const AT* part, int nblk, int npfK, AT* raw) {
+__global__ void __launch_bounds__(256) k_reduce_pf(const float* part, int nblk, int npfK, float* raw) {
     __shared__ double red[8][33];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int i = blockIdx.x * 32 + lane;
@@ -152,16 +151,16 @@ __global__ void __launch_bounds__(256) k_reduce_pf(const AT* part, int nblk, int
         double t = 0.0;
 #pragma unroll
         for (int j = 0; j < 8; ++j) t += red[j][lane];
-        if (i < npfK) raw[i] = (AT)t;
+        if (i < npfK) raw[i] = (float)t;
     }
 }
 
-// raw pass result for parameter k and vector kk, divided by n_s (in AT)
-template <typename AT, typename VT, int K>
-__device__ __forceinline__ AT fin_raw(const FinArgs<AT, VT>& a, int64_t k, int kk) {
+// raw pass result for parameter k and vector kk, divided by n_s
+template <int K>
+__device__ __forceinline__ float fin_raw(const FinArgs& a, int64_t k, int kk) {
     const DevProblem& pb = a.pb;
-    const AT raw = k < pb.ncp ? a.corr_raw[k * K + kk] * a.invC[k] : a.pf_raw[(k - pb.ncp) * K + kk];
-    return raw * (AT)a.inv_n;
+    const float raw = k < pb.ncp ? a.corr_raw[k * K + kk] * a.invC[k] : a.pf_raw[(k - pb.ncp) * K + kk];
+    return raw * (float)a.inv_n;
 }
 
 // Vector kernels cover kVecUnroll elements per thread, strided by the grid,
@@ -171,9 +170,10 @@ constexpr int kVecUnroll = 4;
 
 // out = raw - Obar (Obar . V) + shift V; dot_part = partial out . V.  A
 // centered pass (t_s - Obar . V scattered) already holds the covariance and
-// skips the Obar term.  Element arithmetic in AT, partial dots in FP64.
-template <typename AT, typename VT, int K>
-__global__ void __launch_bounds__(256) k_finalize_S(FinArgs<AT, VT> a) {
+// skips the Obar term.  Element arithmetic in FP32, partial dots in FP64.
+// (Passes with FP64 sums: k_sr_finish.)
+template <int K>
+__global__ void __launch_bounds__(256) k_finalize_S(FinArgs a) {
     if (a.stop && *a.stop) return;
     __shared__ double obv[K];
     if (threadIdx.x < 32) {
@@ -184,43 +184,44 @@ __global__ void __launch_bounds__(256) k_finalize_S(FinArgs<AT, VT> a) {
         }
     }
     __syncthreads();
-    AT ov[K];
+    float ov[K];
 #pragma unroll
-    for (int kk = 0; kk < K; ++kk) ov[kk] = (AT)obv[kk];
-    const AT shift = (AT)a.shift;
+    for (int kk = 0; kk < K; ++kk) ov[kk] = (float)obv[kk];
+    const float shift = (float)a.shift;
     const int64_t nv = a.pb.nv;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     double dl[K];
 #pragma unroll
     for (int kk = 0; kk < K; ++kk) dl[kk] = 0.0;
     for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < nv; i0 += kVecUnroll * stride) {
-        AT ob[kVecUnroll], v[kVecUnroll][K], raw[kVecUnroll][K];
+        float ob[kVecUnroll], v[kVecUnroll][K], raw[kVecUnroll][K];
 #pragma unroll
         for (int u = 0; u < kVecUnroll; ++u) {
             const int64_t k = i0 + u * stride;
-            ob[u] = AT(0);
+            ob[u] = 0.f;
 #pragma unroll
-            for (int kk = 0; kk < K; ++kk) v[u][kk] = raw[u][kk] = AT(0);
+            for (int kk = 0; kk < K; ++kk) v[u][kk] = raw[u][kk] = 0.f;
             if (k < nv) {
-                if (!a.centered) ob[u] = a.ObarA[k];
+                if (!a.centered) ob[u] = a.Obar[k];
 #pragma unroll
                 for (int kk = 0; kk < K; ++kk) {
-                    v[u][kk] = (AT)a.V[kk * nv + k];
-                    raw[u][kk] = fin_raw<AT, VT, K>(a, k, kk);
+                    v[u][kk] = a.V[kk * nv + k];
+                    raw[u][kk] = fin_raw<K>(a, k, kk);
                 }
             }
         }
-        AT part[K];
+        float part[K];
 #pragma unroll
-        for (int kk = 0; kk < K; ++kk) part[kk] = AT(0);
+        for (int kk = 0; kk < K; ++kk) part[kk] = 0.f;
 #pragma unroll
         for (int u = 0; u < kVecUnroll; ++u) {
             const int64_t k = i0 + u * stride;
             if (k < nv) {
 #pragma unroll
                 for (int kk = 0; kk < K; ++kk) {
-                    const AT o = raw[u][kk] - ob[u] * ov[kk] + shift * v[u][kk];
-                    a.out[kk * nv + k] = (VT)o;
+                    const float o = raw[u][kk] - ob[u] * ov[kk] + shift * v[u][kk];
+                    if (a.out64) a.out64[kk * nv + k] = (double)o;
+                    else a.out[kk * nv + k] = o;
                     part[kk] += o * v[u][kk];
                 }
             }
@@ -229,24 +230,6 @@ __global__ void __launch_bounds__(256) k_finalize_S(FinArgs<AT, VT> a) {
         for (int kk = 0; kk < K; ++kk) dl[kk] += (double)part[kk];
     }
     if (a.dot_part) block_reduce_store<K>(dl, a.dot_part);
-}
-
-// gradient mode: K = 2 with t_s = (1, E_s)
-template <typename AT>
-__global__ void __launch_bounds__(256) k_finalize_grad(FinArgs<AT, double> a) {
-    __shared__ double em;
-    if (threadIdx.x < 32) {
-        double s = warp_sum_partials(a.E_sum, a.n_E_part, 0, 1);
-        if (threadIdx.x == 0) em = s * a.inv_n;
-    }
-    __syncthreads();
-    const int64_t nv = a.pb.nv;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nv; k += (int64_t)gridDim.x * blockDim.x) {
-        double o = fin_raw<AT, double, 2>(a, k, 0);
-        double eo = fin_raw<AT, double, 2>(a, k, 1);
-        a.Obar_out[k] = o;
-        a.g_out[k] = eo - em * o;
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -283,6 +266,40 @@ __global__ void __launch_bounds__(256) k_dot_part(const TA* x, const TB* y, int6
         for (int u = 0; u < kVecUnroll; ++u)
 #pragma unroll
             for (int kk = 0; kk < K; ++kk) loc[kk] += xv[u] * yv[u][kk];
+    }
+    block_reduce_store<K>(loc, part);
+}
+
+// What a product with FP32 sums needs first, in one launch instead of a cast, a
+// memset and k_dot_part (with the widening in k_finalize_S, 240 -> 211 us a product
+// on the 8x8 lattice with 65,536 BF16 samples, 139 -> 116 us for four vectors on 6x6).
+template <int K>
+__global__ void __launch_bounds__(256) k_cast_dot(const double* src, float* dst, const double* Obar, int64_t n, double* part,
+                                                  float* clear, int64_t nclear) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x, t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (int64_t i = t0; i < nclear; i += stride) clear[i] = 0.f;
+    double loc[K];
+#pragma unroll
+    for (int kk = 0; kk < K; ++kk) loc[kk] = 0.0;
+    for (int64_t i0 = t0; i0 < n; i0 += kVecUnroll * stride) {
+        double xv[kVecUnroll];
+        float yv[kVecUnroll][K];
+#pragma unroll
+        for (int u = 0; u < kVecUnroll; ++u) {
+            const int64_t i = i0 + u * stride;
+            xv[u] = i < n ? Obar[i] : 0.0;
+#pragma unroll
+            for (int kk = 0; kk < K; ++kk) yv[u][kk] = i < n ? (float)src[kk * n + i] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < kVecUnroll; ++u) {
+            const int64_t i = i0 + u * stride;
+#pragma unroll
+            for (int kk = 0; kk < K; ++kk) {
+                if (i < n) dst[kk * n + i] = yv[u][kk];
+                loc[kk] += xv[u] * (double)yv[u][kk];
+            }
+        }
     }
     block_reduce_store<K>(loc, part);
 }
@@ -749,15 +766,12 @@ template __global__ void k_corr_scatter<double, 4>(CorrArgs<double>);
 template __global__ void k_corr_scatter<float, 1>(CorrArgs<float>);
 template __global__ void k_corr_scatter<float, 2>(CorrArgs<float>);
 template __global__ void k_corr_scatter<float, 4>(CorrArgs<float>);
-template __global__ void k_finalize_S<double, double, 1>(FinArgs<double, double>);
-template __global__ void k_finalize_S<double, double, 2>(FinArgs<double, double>);
-template __global__ void k_finalize_S<double, double, 4>(FinArgs<double, double>);
-template __global__ void k_finalize_S<float, float, 1>(FinArgs<float, float>);
-template __global__ void k_finalize_S<float, float, 2>(FinArgs<float, float>);
-template __global__ void k_finalize_S<float, float, 4>(FinArgs<float, float>);
-template __global__ void k_finalize_grad<double>(FinArgs<double, double>);
-template __global__ void k_reduce_pf<double>(const double*, int, int, double*);
-template __global__ void k_reduce_pf<float>(const float*, int, int, float*);
+template __global__ void k_finalize_S<1>(FinArgs);
+template __global__ void k_cast_dot<1>(const double*, float*, const double*, int64_t, double*, float*, int64_t);
+template __global__ void k_finalize_S<2>(FinArgs);
+template __global__ void k_cast_dot<2>(const double*, float*, const double*, int64_t, double*, float*, int64_t);
+template __global__ void k_finalize_S<4>(FinArgs);
+template __global__ void k_cast_dot<4>(const double*, float*, const double*, int64_t, double*, float*, int64_t);
 template __global__ void k_dot_part<double, double, 1>(const double*, const double*, int64_t, double*, const int*);
 template __global__ void k_dot_part<double, double, 2>(const double*, const double*, int64_t, double*, const int*);
 template __global__ void k_dot_part<double, double, 4>(const double*, const double*, int64_t, double*, const int*);
