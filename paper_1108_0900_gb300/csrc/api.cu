@@ -2734,7 +2734,7 @@ static int lm_launch(vmc_ctx* h, const double* x, double* Hx, double* Sx, const 
     a.tables = (size_t)a.L.bytes + 64 <= h->smem_optin && h->lm_max_list <= 64;
     if (!a.tables) a.L = layout(false);
     const size_t smem = (size_t)a.L.bytes;
-    if (smem + 64 > h->smem_optin) {
+    if (smem + 16 > h->smem_optin) {
         set_err("linear-method product: per-sample workspace exceeds shared memory");
         return VMC_ERR_UNSUPPORTED;
     }

@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(256) k_sv_finish(SortedArgs a, const float* pf
 // shared memory of one sample: elements of R from the start, then bytes
 struct LmLayout {
     int X, G, Xo, Pm, D, Y, w, cold, rcm, fr, fx;
-    int ev_bytes, cidx_bytes, occ_bytes, bytes;
+    int cidx_bytes, occ_bytes, bytes;
 };
 LmLayout lm_layout(int ns, int nu, int nd, int n_mu, int ncorr, int nentry, int elem, bool tables);
 

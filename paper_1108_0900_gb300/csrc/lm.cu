@@ -47,6 +47,7 @@
 // took 47.4 ms.  4x4 lattice, 2x2 correlators, 4,097 samples, FP64: 0.35 ms,
 // 0.57 before.  Threads x CTAs per SM by registers, FP32: 128 x 4 8.1, x 6 7.5,
 // x 8 6.7 ms; 256 threads 11.4, 8.6, 7.3 ms.
+#include <algorithm>
 #include "ansatz.cuh"
 #include "common.cuh"
 #include "kernels.h"
@@ -202,14 +203,13 @@ LmLayout lm_layout(int ns, int nu, int nd, int n_mu, int ncorr, int nentry, int 
     L.w = L.Y + ns * ns;
     L.cold = L.w + n_mu;
     L.rcm = L.cold + ncorr;
-    L.fr = L.rcm + nex;
+    L.rcm = even(L.rcm);
+    L.fr = L.rcm + std::max(nex, 2 * ns * 8 / elem);   // the ratios' place takes the event sums later
     L.fx = L.fr + (tables ? 2 * nentry : 0);
     const int n = even(L.fx + (tables ? 2 * nentry : 0));
-    // doubles (event sums of the pair correlators), then states and orbitals
-    L.ev_bytes = n * elem;
-    L.cidx_bytes = L.ev_bytes + 2 * ns * 8;
+    L.cidx_bytes = n * elem;
     L.occ_bytes = L.cidx_bytes + ncorr * 4;
-    L.bytes = (L.occ_bytes + 64 + 3 * 128 + 15) / 16 * 16;
+    L.bytes = (L.occ_bytes + N + E + 4 * ns + 15) / 16 * 16;
     return L;
 }
 
@@ -251,12 +251,12 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 3) k_lm_apply(LmArgs
     R *w = tab + L.w, *cold = tab + L.cold;   // old-state adjoint sums per correlator
     R* rcm = tab + L.rcm;                // correlator ratio of every move
     R *fr = a.tables ? tab + L.fr : nullptr, *fx = tab + L.fx;   // see corr_ratio_dir
-    double* ev = (double*)(smem + L.ev_bytes);   // sum of the coefficients of every spin orbital's moves
+    double* ev = (double*)rcm;           // then: sum of the coefficients of every spin orbital's moves
     uint32_t* cidx = (uint32_t*)(smem + L.cidx_bytes);
     uint8_t* occ = smem + L.occ_bytes;
-    uint8_t* emp = occ + 64;
-    int8_t* opos = (int8_t*)(emp + 128);   // position of an occupied orbital, or
-    int8_t* epos = opos + 128;             // of an empty one (else -1)
+    uint8_t* emp = occ + N;
+    int8_t* opos = (int8_t*)(emp + E);   // position of an occupied orbital, or
+    int8_t* epos = opos + M;             // of an empty one (else -1)
     const R* Xt = (const R*)a.Xt;
     const R* xc = (const R*)a.xc;
     const R* Lval = (const R*)a.Lval;
@@ -290,7 +290,6 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 3) k_lm_apply(LmArgs
             opos[o] = on ? (int8_t)r : (int8_t)-1;
             epos[o] = on ? (int8_t)-1 : (int8_t)r;
             if (!on) emp[r] = (uint8_t)o;
-            ev[o] = 0.0;
         }
         for (int e = tid; e < pb.P; e += bd) {
             const uint16_t t = pb.pairtab[e];
