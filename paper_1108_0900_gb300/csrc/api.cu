@@ -810,6 +810,13 @@ static int read_status(vmc_ctx* h, cudaStream_t st) {
     return VMC_OK;
 }
 
+// warps per CTA of the kernels with a warp per walker or sample: four, or fewer
+// where that would leave SMs idle (4x4 lattice, 64 FP64 chains: 4,232 us with four
+// warps on each of 16 SMs, 4,143 us with one on each of 64)
+static int spread_warps(const vmc_ctx* h, int64_t n) {
+    return (int)std::max<int64_t>(1, std::min<int64_t>(4, (n + h->nsm - 1) / h->nsm));
+}
+
 // fills the problem-dependent fields of `a` (strides, shared-memory slice per
 // walker) and returns the slice size
 static size_t prep_walkers(vmc_ctx* h, SampleArgs& a, bool fp64) {
@@ -828,8 +835,8 @@ static size_t prep_walkers(vmc_ctx* h, SampleArgs& a, bool fp64) {
 
 static int launch_walkers(vmc_ctx* h, SampleArgs& a, bool fp64, cudaStream_t st) {
     if (fp64 && a.props_per_sweep == 0) {
-        // given configurations, FP64 from scratch: four warps (samples) per CTA, or fewer
-        int warps = 4;
+        // given configurations, FP64 from scratch
+        int warps = spread_warps(h, a.n_walkers);
         while (warps > 1 && measure64_smem(h->N, h->P, h->ncorr, warps) > h->smem_optin) warps /= 2;
         const size_t smem = measure64_smem(h->N, h->P, h->ncorr, warps);
         if (smem > h->smem_optin) return VMC_ERR_UNSUPPORTED;
@@ -842,7 +849,7 @@ static int launch_walkers(vmc_ctx* h, SampleArgs& a, bool fp64, cudaStream_t st)
         return VMC_OK;
     }
     const size_t wb = prep_walkers(h, a, fp64);
-    int wpb = (int)std::min<size_t>(4, h->smem_optin / wb);
+    int wpb = (int)std::min<size_t>(spread_warps(h, a.n_walkers), h->smem_optin / wb);
     if (wpb < 1) return VMC_ERR_UNSUPPORTED;
     size_t smem = wb * wpb;
     int blocks = (a.n_walkers + wpb - 1) / wpb;
@@ -1031,7 +1038,7 @@ extern "C" int vmc_sample_batch(const vmc_handle* hs, int n, int n_burn, const u
         wb = std::max(wb, prep_walkers(hs[b], args[b], fp64));
         wstart[b + 1] = wstart[b] + hs[b]->n_walkers;
     }
-    const int wpb = (int)std::min<size_t>(4, h0->smem_optin / wb);
+    const int wpb = (int)std::min<size_t>(spread_warps(h0, wstart[n]), h0->smem_optin / wb);
     if (wpb < 1) return VMC_ERR_UNSUPPORTED;
     void* dbuf = nullptr;
     const size_t abytes = round_up(sizeof(SampleArgs) * n, 256);
@@ -1186,7 +1193,7 @@ extern "C" int vmc_logpsi(vmc_handle h, double* out, void* stream) {
     a.s_cidx = h->d_cidx; a.ncst = h->ncst;
     a.fulltab = h->d_fulltab;
     a.out = out;
-    const int wpb = 4;
+    const int wpb = spread_warps(h, h->n_s);
     const size_t smem = measure64_smem(h->N, h->P, 0, wpb);
     VCK(cudaFuncSetAttribute(k_logpsi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     k_logpsi<<<(unsigned)((h->n_s + wpb - 1) / wpb), 32 * wpb, smem, st>>>(a); h->n_launch++;
