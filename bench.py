@@ -109,7 +109,7 @@ PASS_KERNELS = {"sorted": "k_gather_G<1,U> + k_scatter_T<1> (sorted two-pass Eq.
                 "compact": "k_gather_C<U> + k_scatter_T<1> (two-pass Eq. 7 product, compact gather, BF16 store)",
                 "fused": "k_sv_fused<U> + k_sv_finish (fused single-pass Eq. 7 product, BF16 store)",
                 "staged": "k_sr_stream<bf16,1> + k_corr_scatter + k_reduce_pf (staged per-sample pass)",
-                "generic": "k_sr_main<bf16,float,1> + k_corr_scatter + k_reduce_pf (generic per-sample pass)"}
+                "generic": "k_sr_main<bf16,1> + k_corr_scatter + k_reduce_pf (generic per-sample pass)"}
 # nominal FP64 (non-tensor) rate of one GB300 (the peaks file measures no FP64)
 FP64_PEAK_TFLOPS = 1.25
 AUTOTUNE_CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "paper_1108_0900_gb300", "_build",
@@ -360,7 +360,7 @@ def run_gpu(args, rank, world, dist):
                 "cg_iterations": float(np.mean([i["iterations"] for i in infos64])),
                 "true_rel_residual": max(i["true_rel_residual"] for i in infos64),
                 "converged": all(i["converged"] for i in infos64),
-                "roofline": {"bound": "alu", "kernel": "k_sr_main<double,double,1> (FP64 store, FP64 FMA)",
+                "roofline": {"bound": "alu", "kernel": "k_sr_pass<double,1> (FP64 store, FP64 FMA)",
                              "product_ms": round(ms_p64, 4),
                              "achieved": round(2 * fma / (ms_p64 * 1e-3) / 1e12, 3), "unit": "TFLOP/s",
                              "peak": FP64_PEAK_TFLOPS, "peak_kind": "nominal FP64 rate of the GB300",

@@ -10,7 +10,9 @@
 // synchronisation is one barrier per tile between gather and scatter.  There
 // are as many images as shared memory holds (two at 128 spin orbitals, one
 // per warp on small lattices, where a warp keeps its sample for both halves
-// and needs no barrier).  The sums have a fixed order.
+// and needs no barrier).  The sums have a fixed order.  Small correlator blocks
+// enter the images too (in FP64, a warp's lanes over the correlators); larger ones
+// are summed from the t_s by a kernel of their own.
 //
 // What bounds it: the FP64 store's pass the FP64 pipe (two FMAs per element, 72 %
 // busy), the FP32 store's issue slots and shared-memory latency (32 warps).  8x8

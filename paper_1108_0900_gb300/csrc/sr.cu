@@ -1,7 +1,7 @@
-// SR kernels over the stored derivative ratios (Sec. II.A):
+// SR kernels over the stored derivative ratios (Sec. II.A) with FP32 sums (FP64 sums
+// and the gradient: pass.cu):
 //   - the matrix-free product of Eq. 7, (1/n_s) sum_s O_s (O_s . v), with the
 //     covariance term -Obar (Obar . v) and the absolute shift eps v;
-//   - the sample means Obar, <E_L> and the gradient g = <E_L O> - <E_L> Obar;
 //   - the vector updates of conjugate gradient with FP64 scalars.
 //
 // Per sample the O vector is sparse: correlator c contributes 1/C at its own
