@@ -773,10 +773,7 @@ template __global__ void k_cast_dot<2>(const double*, float*, const double*, int
 template __global__ void k_finalize_S<4>(FinArgs);
 template __global__ void k_cast_dot<4>(const double*, float*, const double*, int64_t, double*, float*, int64_t);
 template __global__ void k_dot_part<double, double, 1>(const double*, const double*, int64_t, double*, const int*);
-template __global__ void k_dot_part<double, double, 2>(const double*, const double*, int64_t, double*, const int*);
-template __global__ void k_dot_part<double, double, 4>(const double*, const double*, int64_t, double*, const int*);
 template __global__ void k_dot_part<double, float, 1>(const double*, const float*, int64_t, double*, const int*);
-template __global__ void k_dot_part<double, float, 2>(const double*, const float*, int64_t, double*, const int*);
 template __global__ void k_dot_part<double, float, 4>(const double*, const float*, int64_t, double*, const int*);
 template __global__ void k_cast<float>(const double*, float*, int64_t, double);
 template __global__ void k_cast<double>(const double*, double*, int64_t, double);
