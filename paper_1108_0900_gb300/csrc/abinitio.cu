@@ -521,7 +521,7 @@ __global__ void __launch_bounds__(kAbThreads, sizeof(R) == 4 ? 5 : 3) k_ab_energ
         const R* Xs = (const R*)a.X + s * N * N;
         for (int t = tid; t < N * N; t += bd) X[(t / N) * XS + t % N] = Xs[t];
         __syncthreads();
-        // G: a warp's lanes over the electrons, four holes per pass over X; the
+        // G: a warp's lanes over the electrons (W per lane), four holes per pass over X; the
         // lanes hold the holes' F rows and hand them round by shuffle
         for (int h0 = 4 * wid; h0 < E; h0 += 4 * nw) {
             R acc[4][2];
@@ -669,7 +669,8 @@ __global__ void __launch_bounds__(kAbThreads, sizeof(R) == 4 ? 5 : 3) k_ab_energ
 
 template <typename R>
 static cudaError_t launch_ab(const AbArgs& a, int threads, size_t smem, int nsm, cudaStream_t st) {
-    auto kern = a.pb.ns <= 32 ? k_ab_energy<R, 1> : k_ab_energy<R, 2>;
+    // a lane takes W sites (mixed doubles) and W electrons (rows of G)
+    auto kern = a.pb.ns <= 32 && a.pb.N <= 32 ? k_ab_energy<R, 1> : k_ab_energy<R, 2>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int per = 0;
