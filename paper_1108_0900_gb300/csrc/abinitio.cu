@@ -493,8 +493,9 @@ __global__ void __launch_bounds__(kAbThreads, sizeof(R) == 4 ? 5 : 3) k_ab_energ
     const uint64_t smask = (ns == 64) ? ~0ull : ((1ull << ns) - 1ull);
 
     for (int64_t s = blockIdx.x; s < a.n_s; s += gridDim.x) {
-        // configuration; a sample that was not written (its walker failed) is
-        // left alone, the walker has set the status
+        // configuration; a sample that was never written (its walker failed) is
+        // left alone, the walker has set the status; positions and correlator
+        // states are written together, so where the positions hold, so do the states
         uint64_t up = 0, dn = 0;
         bool bad = false;
         for (int i = 0; i < N; ++i) {

@@ -143,7 +143,7 @@ struct vmc_ctx {
     double* d_pf64 = nullptr;
     char* d_abX = nullptr;       // ab initio: [ncap][N][N] pairing inverses for the local energy's pass
     size_t abX_bytes = 0;
-    uint8_t* d_abpos = nullptr;  // [ncap][Nst] the orbitals at their positions
+    uint8_t* d_abpos = nullptr;  // [ncap][Nst] the orbitals at their positions (0xFF: never written)
     float* d_pf32 = nullptr;
     __nv_bfloat16* d_pf16 = nullptr;
     double* d_Obar[3] = {nullptr, nullptr, nullptr};
@@ -574,6 +574,14 @@ extern "C" int vmc_create(const vmc_lattice* lat, const vmc_hamiltonian* ham, co
     ACK(h->alloc(&h->d_lnrun, h->ncap));
     if (h->fp64_refresh) ACK(h->alloc(&h->d_Echain, h->ncap));
     if (h->keep64) ACK(h->alloc(&h->d_pf64, (size_t)h->ncap * h->Pst));
+    if (h->ham == VMC_ABINITIO) {
+        // no orbital at any position: a sample that a failed walker never wrote is
+        // passed over by the local energy's pass, which would index the amplitudes
+        // with whatever its correlator states held (vmc_set_params, which comes before
+        // any sample, waits for this)
+        ACK(h->alloc(&h->d_abpos, (size_t)h->ncap * h->Nst));
+        if (cudaMemset(h->d_abpos, 0xFF, (size_t)h->ncap * h->Nst) != cudaSuccess) return fail(VMC_ERR_CUDA);
+    }
     {
         std::vector<uint32_t> ft;
         const int Puu = nu * (nu - 1) / 2, Pdd = nd * (nd - 1) / 2;
@@ -883,7 +891,6 @@ static int store_targets(vmc_ctx* h, SampleArgs& a, bool fp64) {
             VCK(h->alloc(&h->d_abX, bytes));
             h->abX_bytes = bytes;
         }
-        if (!h->d_abpos) VCK(h->alloc(&h->d_abpos, (size_t)h->ncap * h->Nst));
         a.s_X = h->d_abX;
         a.s_pos = h->d_abpos;
     }
