@@ -151,7 +151,12 @@ typedef struct {
 
 /* Create a handle on the current CUDA device.  Copies every input.  Errors:
  * INVALID_ARG (sizes out of range, odd N, > 64 sites, bad bond or site index),
- * OOM, CUDA. */
+ * OOM, CUDA.  Device memory is taken here for n_walkers x samples_per_walker
+ * samples; sampling and measuring take none.  An ab initio handle holds, beside
+ * its stores, the N x N pairing inverses between the walkers and the local
+ * energies: N^2 values of the walkers' precision per sample, 2 GiB at most
+ * (larger sets are sampled and measured in pieces, with the same results), but
+ * one walker's samples at least. */
 int vmc_create(const vmc_lattice* lat, const vmc_hamiltonian* ham, const vmc_ansatz* ans,
                const vmc_options* opt, vmc_handle* out);
 int vmc_destroy(vmc_handle h);

@@ -16,6 +16,9 @@ namespace {
 
 constexpr int kMaxK = 4;
 constexpr int kNumPart = 256;   // blocks of the reduction kernels
+// ab initio: bytes of pairing inverses between the walkers and the local energy's pass;
+// larger sample sets go through it in pieces (65,536 samples of 64 electrons in FP64)
+constexpr size_t kAbWork = (size_t)2 << 30;
 constexpr int kChunk = 16;      // CG iterations between host convergence checks
 constexpr int kBlockInnerMax = 4096;   // block CG steps of one inner solve at most
 constexpr int kScalX0 = 7;      // d_scal slot of the SR update's x_0
@@ -141,8 +144,9 @@ struct vmc_ctx {
     unsigned char* d_batch = nullptr;   // argument blocks of batched launches led by this handle
     size_t batch_bytes = 0;
     double* d_pf64 = nullptr;
-    char* d_abX = nullptr;       // ab initio: [ncap][N][N] pairing inverses for the local energy's pass
+    char* d_abX = nullptr;       // ab initio: [piece][N][N] pairing inverses for the local energy's pass
     size_t abX_bytes = 0;
+    int64_t ab_piece(bool fp64) const { return (int64_t)(abX_bytes / ((size_t)N * N * (fp64 ? 8 : 4))); }   // samples
     uint8_t* d_abpos = nullptr;  // [ncap][Nst] the orbitals at their positions (0xFF: never written)
     float* d_pf32 = nullptr;
     __nv_bfloat16* d_pf16 = nullptr;
@@ -575,6 +579,12 @@ extern "C" int vmc_create(const vmc_lattice* lat, const vmc_hamiltonian* ham, co
     if (h->fp64_refresh) ACK(h->alloc(&h->d_Echain, h->ncap));
     if (h->keep64) ACK(h->alloc(&h->d_pf64, (size_t)h->ncap * h->Pst));
     if (h->ham == VMC_ABINITIO) {
+        // the inverses of every sample, or kAbWork; those of one walker's samples at
+        // least, and of one sample in FP64 (a handle of FP32 walkers is also measured
+        // in FP64, in smaller pieces)
+        const size_t nn = (size_t)N * N, one = nn * (h->wprec == VMC_FP64 ? 8 : 4);
+        h->abX_bytes = std::max({std::min(h->ncap * one, kAbWork), h->spw * one, nn * 8});
+        ACK(h->alloc(&h->d_abX, h->abX_bytes));
         // no orbital at any position: a sample that a failed walker never wrote is
         // passed over by the local energy's pass, which would index the amplitudes
         // with whatever its correlator states held (vmc_set_params, which comes before
@@ -868,8 +878,8 @@ static int launch_walkers(vmc_ctx* h, SampleArgs& a, bool fp64, cudaStream_t st)
     return VMC_OK;
 }
 
-// where walkers of the given precision write the O store
-static int store_targets(vmc_ctx* h, SampleArgs& a, bool fp64) {
+// where walkers write the O store
+static void store_targets(vmc_ctx* h, SampleArgs& a) {
     a.s_occ = h->d_socc; a.Nst = h->Nst;
     a.s_cidx = h->d_cidx; a.ncst = h->ncst;
     a.s_E = h->d_E;
@@ -879,39 +889,26 @@ static int store_targets(vmc_ctx* h, SampleArgs& a, bool fp64) {
     a.s_pf16 = h->keeplow ? h->d_pf16 : nullptr;
     a.Pst = h->Pst;
     if (h->ham == VMC_ABINITIO) {
-        // what the local energy's pass reads (FP64 walkers and refreshes: twice the bytes)
-        const size_t bytes = (size_t)h->ncap * h->N * h->N * (fp64 ? 8 : 4);
-        if (h->abX_bytes < bytes) {
-            if (h->d_abX) {
-                VCK(cudaFree(h->d_abX));   // waits for the work that reads it
-                h->allocs.erase(std::find(h->allocs.begin(), h->allocs.end(), (void*)h->d_abX));
-                h->d_abX = nullptr;
-                h->abX_bytes = 0;
-            }
-            VCK(h->alloc(&h->d_abX, bytes));
-            h->abX_bytes = bytes;
-        }
         a.s_X = h->d_abX;
         a.s_pos = h->d_abpos;
     }
-    return VMC_OK;
 }
 
-// E_L of the stored samples of an ab initio problem, from the pairing inverses
-// that walkers of the given precision wrote (the Hubbard energy is the
-// walkers' own).  Four warps per sample; two or one where the tables of a
+// E_L of the stored samples [s0, s0 + n_s) of an ab initio problem, from the
+// pairing inverses that walkers of the given precision wrote (the Hubbard energy
+// is the walkers' own).  Four warps per sample; two or one where the tables of a
 // large FP64 problem leave no room for more, and the general correlator
 // factors where they do not fit at all or correlators span more sites.
-static int ab_energy(vmc_ctx* h, bool fp64, int64_t n_s, cudaStream_t st) {
+static int ab_energy(vmc_ctx* h, bool fp64, int64_t s0, int64_t n_s, cudaStream_t st) {
     if (h->ham != VMC_ABINITIO || n_s == 0) return VMC_OK;
     const size_t rsz = fp64 ? 8 : 4;
     AbArgs a{};
     a.pb = h->pb;
     a.n_s = n_s;
-    a.pos = h->d_abpos; a.Nst = h->Nst;
-    a.s_cidx = h->d_cidx; a.ncst = h->ncst;
+    a.pos = h->d_abpos + s0 * h->Nst; a.Nst = h->Nst;
+    a.s_cidx = h->d_cidx + s0 * h->ncst; a.ncst = h->ncst;
     a.X = h->d_abX;
-    a.s_E = h->d_E;
+    a.s_E = h->d_E + s0;
     a.status = h->status_word();
     const size_t rest = (size_t)h->N * (h->N | 1) * rsz + (size_t)h->ncorr * 4 + 64 + 3 * 128;
     int nw = kAbThreads / 32;
@@ -935,6 +932,30 @@ static int ab_energy(vmc_ctx* h, bool fp64, int64_t n_s, cudaStream_t st) {
     return VMC_OK;
 }
 
+// the store is about to be rewritten: what was built on the old samples goes
+static void drop_built(vmc_ctx* h) {
+    h->obar_ok[0] = h->obar_ok[1] = h->obar_ok[2] = false;
+    h->sorted_ok = h->g_ok = h->corr_ok = false;
+}
+
+// walkers (or given configurations) and, where they write the store, the ab
+// initio energies of their samples: as many walkers at once as the energies'
+// inverses leave room for.  A walker's samples do not depend on the split.
+static int run_walkers(vmc_ctx* h, SampleArgs& a, bool fp64, cudaStream_t st) {
+    if (a.s_occ) drop_built(h);
+    if (!a.s_X) return launch_walkers(h, a, fp64, st);
+    const int64_t all = a.n_walkers, most = std::max<int64_t>(1, h->ab_piece(fp64) / a.spw);
+    const int64_t pieces = (all + most - 1) / most, per = (all + pieces - 1) / pieces;
+    for (int64_t w0 = 0; w0 < all; w0 += per) {
+        a.w0 = (int)w0;
+        a.n_walkers = (int)std::min(per, all - w0);
+        int rc = launch_walkers(h, a, fp64, st);
+        if (!rc) rc = ab_energy(h, fp64, w0 * a.spw, (int64_t)a.n_walkers * a.spw, st);
+        if (rc) return rc;
+    }
+    return VMC_OK;
+}
+
 static int transpose_states(vmc_ctx* h, cudaStream_t st) {
     if (h->ncorr == 0 || h->n_s == 0) return VMC_OK;
     dim3 grid((unsigned)((h->n_s + 31) / 32), (unsigned)((h->ncorr + 31) / 32));
@@ -943,7 +964,7 @@ static int transpose_states(vmc_ctx* h, cudaStream_t st) {
     return VMC_OK;
 }
 
-static int sample_args(vmc_ctx* h, int n_burn, uint64_t seed, SampleArgs& a) {
+static void sample_args(vmc_ctx* h, int n_burn, uint64_t seed, SampleArgs& a) {
     a = SampleArgs{};
     a.n_walkers = h->n_walkers;
     a.spw = h->spw;
@@ -955,7 +976,7 @@ static int sample_args(vmc_ctx* h, int n_burn, uint64_t seed, SampleArgs& a) {
     a.seed = seed;
     a.walker_occ = h->d_wocc;
     a.walker_step = h->d_wstep;
-    return store_targets(h, a, h->wprec == VMC_FP64);
+    store_targets(h, a);
 }
 
 static int after_sampling(vmc_ctx* h, cudaStream_t st);
@@ -965,24 +986,18 @@ extern "C" int vmc_sample(vmc_handle h, int n_burn, uint64_t seed, void* stream)
     if (!h->params_set || !h->walkers_set) return VMC_ERR_STATE;
     cudaStream_t st = (cudaStream_t)stream;
     SampleArgs a;
-    int rc = sample_args(h, n_burn, seed, a);
-    if (rc) return rc;
-    rc = launch_walkers(h, a, h->wprec == VMC_FP64, st);
+    sample_args(h, n_burn, seed, a);
+    int rc = run_walkers(h, a, h->wprec == VMC_FP64, st);
     if (rc) return rc;
     return after_sampling(h, st);
 }
 
-// the store holds a new set of samples: invalidate what was built on the old
-// one, the ab initio energies, refresh in FP64 if asked, transpose the
+// the store holds a new set of samples: refresh in FP64 if asked, transpose the
 // correlator states
 static int after_sampling(vmc_ctx* h, cudaStream_t st) {
     int rc;
     h->n_s = h->ncap;
-    h->obar_ok[0] = h->obar_ok[1] = h->obar_ok[2] = false;
-    h->sorted_ok = h->g_ok = h->corr_ok = false;
     h->refreshed = false;
-    rc = ab_energy(h, h->wprec == VMC_FP64, h->n_s, st);
-    if (rc) return rc;
     if (h->wprec == VMC_FP32 && h->fp64_refresh) {
         // FP64 refresh of every stored sample: the pairing inverse, E_L and O
         // from scratch in FP64, rounded into the stores; the chains' own E_L
@@ -994,11 +1009,9 @@ static int after_sampling(vmc_ctx* h, cudaStream_t st) {
         m.spw = 1;
         m.want_energy = 1;
         m.walker_occ = h->d_mocc;
-        rc = store_targets(h, m, true);
-        if (rc) return rc;
+        store_targets(h, m);
         m.s_lnrun = nullptr;   // keep the chains' running log-amplitudes
-        rc = launch_walkers(h, m, true, st);
-        if (!rc) rc = ab_energy(h, true, h->n_s, st);
+        rc = run_walkers(h, m, true, st);
         if (rc) return rc;
         h->refreshed = true;
     }
@@ -1039,14 +1052,25 @@ extern "C" int vmc_sample_batch(const vmc_handle* hs, int n, int n_burn, const u
     std::vector<SampleArgs> args(n);
     std::vector<int> wstart(n + 1, 0);
     size_t wb = 0;
+    bool split = false;   // some problem's samples do not fit its energies' workspace
     for (int b = 0; b < n; ++b) {
-        int rs = sample_args(hs[b], n_burn, seeds[b], args[b]);
-        if (rs) return rs;
+        sample_args(hs[b], n_burn, seeds[b], args[b]);
+        split = split || (args[b].s_X && hs[b]->ab_piece(fp64) < hs[b]->ncap);
         wb = std::max(wb, prep_walkers(hs[b], args[b], fp64));
         wstart[b + 1] = wstart[b] + hs[b]->n_walkers;
     }
     const int wpb = (int)std::min<size_t>(spread_warps(h0, wstart[n]), h0->smem_optin / wb);
     if (wpb < 1) return VMC_ERR_UNSUPPORTED;
+    if (split) {   // one after another, each in its pieces
+        int first = VMC_OK;
+        for (int b = 0; b < n; ++b) {
+            int rc = run_walkers(hs[b], args[b], fp64, st);
+            if (!rc) rc = after_sampling(hs[b], st);
+            if (rc && !first) first = rc;
+        }
+        return first;
+    }
+    for (int b = 0; b < n; ++b) drop_built(hs[b]);
     void* dbuf = nullptr;
     const size_t abytes = round_up(sizeof(SampleArgs) * n, 256);
     int rc = batch_buffer(h0, abytes + sizeof(int) * (n + 1), &dbuf);
@@ -1063,7 +1087,8 @@ extern "C" int vmc_sample_batch(const vmc_handle* hs, int n, int n_burn, const u
     VCK(cudaStreamSynchronize(st));
     int first = VMC_OK;
     for (int b = 0; b < n; ++b) {
-        rc = after_sampling(hs[b], st);
+        rc = ab_energy(hs[b], fp64, 0, hs[b]->ncap, st);
+        if (!rc) rc = after_sampling(hs[b], st);
         if (rc && !first) first = rc;
     }
     return first;
@@ -1080,12 +1105,10 @@ static int measure_device_configs(vmc_ctx* h, int64_t n_s, bool fp64, const doub
     a.want_energy = bgrad ? 0 : 1;
     a.walker_occ = h->d_mocc;
     a.walker_step = nullptr;
-    int rc = to_store ? store_targets(h, a, fp64) : VMC_OK;
-    if (rc) return rc;
+    if (to_store) store_targets(h, a);
     a.bw = bw;
     a.bgrad = bgrad;
-    rc = launch_walkers(h, a, fp64, st);
-    return rc || !to_store ? rc : ab_energy(h, fp64, n_s, st);
+    return run_walkers(h, a, fp64, st);
 }
 
 extern "C" int vmc_measure(vmc_handle h, const uint8_t* occ, int64_t n_s, void* stream) {
@@ -1098,8 +1121,6 @@ extern "C" int vmc_measure(vmc_handle h, const uint8_t* occ, int64_t n_s, void* 
     rc = measure_device_configs(h, n_s, h->wprec == VMC_FP64, nullptr, nullptr, true, st);
     if (rc) return rc;
     h->n_s = n_s;
-    h->obar_ok[0] = h->obar_ok[1] = h->obar_ok[2] = false;
-    h->sorted_ok = h->g_ok = h->corr_ok = false;
     rc = transpose_states(h, st);
     if (rc) return rc;
     return read_status(h, st);
@@ -1219,8 +1240,6 @@ extern "C" int vmc_logpsi_backward(vmc_handle h, const double* w, double* grad, 
         rc = measure_device_configs(h, h->n_s, true, w, grad, false, st);
     } else {
         rc = measure_device_configs(h, h->n_s, true, nullptr, nullptr, true, st);
-        h->obar_ok[0] = h->obar_ok[1] = h->obar_ok[2] = false;
-    h->sorted_ok = h->g_ok = h->corr_ok = false;
     }
     if (rc) return rc;
     return read_status(h, st);

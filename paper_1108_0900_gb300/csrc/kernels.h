@@ -13,6 +13,7 @@ namespace vmc {
 struct SampleArgs {
     DevProblem pb;
     int n_walkers;        // warps launched (walkers or given configurations)
+    int w0;               // the first one's number
     int spw;              // measurements per walker
     int n_burn;           // sweeps before the first measurement
     int props_per_sweep;  // N for sampling, 0 to only measure
@@ -36,7 +37,7 @@ struct SampleArgs {
     float* s_pf32;
     __nv_bfloat16* s_pf16;
     int64_t Pst;
-    void* s_X;            // [n_s][N][N] the pairing inverse in the walker's precision (may be null)
+    void* s_X;            // [n_s][N][N] the pairing inverse in the walker's precision (may be null), from sample w0 spw on
     uint8_t* s_pos;       // [n_s][Nst] the orbitals at its positions
     // adjoint mode: bgrad[k] += bw[s] O_k(n_s) instead of writing the store
     const double* bw;

@@ -166,8 +166,9 @@ __global__ void __launch_bounds__(128) k_measure64(SampleArgs a, const uint32_t*
     double* A = (double*)(cd + scratch_pairs(N));
     uint32_t* cidx = (uint32_t*)(A + P + (P & 1));
     uint8_t* occ = (uint8_t*)(cidx + pb.ncorr);
-    const int64_t s = (int64_t)blockIdx.x * (blockDim.x >> 5) + wid;
-    if (s >= a.n_walkers) return;
+    const int64_t t0 = (int64_t)blockIdx.x * (blockDim.x >> 5) + wid;
+    if (t0 >= a.n_walkers) return;
+    const int64_t s = a.w0 + t0;
 
     // ---- the configuration --------------------------------------------------
     uint64_t up = 0, dn = 0;
@@ -286,7 +287,7 @@ __global__ void __launch_bounds__(128) k_measure64(SampleArgs a, const uint32_t*
         return;
     }
     if (a.s_X) {   // the whole inverse, for the ab initio energy's pass
-        double* dst = (double*)a.s_X + s * N * N;
+        double* dst = (double*)a.s_X + t0 * N * N;
         for (int t = lane; t < N * N; t += 32) dst[t] = t / N == t % N ? 0.0 : get(A, N, t / N, t % N);
         for (int i = lane; i < N; i += 32) a.s_pos[s * a.Nst + i] = occ[i];
     }

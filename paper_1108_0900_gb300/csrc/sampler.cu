@@ -448,7 +448,7 @@ __device__ void walker_run(const SampleArgs& a, int w, unsigned char* base) {
         }
         __syncwarp();
         if (a.s_X) {   // the whole inverse and its positions' orbitals, for the ab initio energy's pass
-            R* dst = (R*)a.s_X + s * N * N;
+            R* dst = (R*)a.s_X + (s - (int64_t)a.w0 * a.spw) * N * N;
             for (int t = lane; t < N * N; t += 32) dst[t] = X[(t / N) * XS + t % N];
             for (int i = lane; i < N; i += 32) a.s_pos[s * a.Nst + i] = pos_orb[i];
         }
@@ -480,7 +480,7 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 5 : 4) k_walkers(SampleA
     const int wid = threadIdx.x >> 5;
     const int w = blockIdx.x * (blockDim.x >> 5) + wid;
     if (w >= a.n_walkers) return;
-    walker_run<R>(a, w, smem_raw + (size_t)wid * a.warp_bytes);
+    walker_run<R>(a, a.w0 + w, smem_raw + (size_t)wid * a.warp_bytes);
 }
 
 // Several problems (lattices of uneven size) in one launch: warp g runs

@@ -1,5 +1,5 @@
 """The ab initio local energy where a short cut would show: more electrons than a warp
-has lanes, samples that no walker wrote.
+has lanes, samples that no walker wrote, sample sets larger than the workspace.
 """
 import numpy as np
 import pytest
@@ -9,7 +9,7 @@ from paper_1108_0900_gb300 import inputs
 from paper_1108_0900_gb300 import vmcsr as V
 from test_gpu_abinitio_energy import condition, energies, problem
 
-pytest.importorskip("torch")
+torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
@@ -50,3 +50,57 @@ def test_samples_that_no_walker_wrote_are_passed_over(prec):
     E = V.vmc_get_samples(h)[1]
     h.close()
     assert np.array_equal(E[~bad], energies(wl, cfgs[~bad], prec))
+
+
+@pytest.mark.parametrize("refresh", [False, True])
+def test_sampling_takes_no_device_memory(refresh):
+    """What sampling and measuring need is there when the handle is."""
+    wl = problem(12, 6, 6, "pairs")
+    occ = inputs.draw_configs(np.random.default_rng(1), 2048, 12, 6, 6)
+
+    def free_before_and_after():
+        h = V.vmc_create(wl, n_walkers=2048, samples_per_walker=4, walker_precision=V.VMC_FP32, fp64_refresh=refresh)
+        V.vmc_set_params(h, wl.C, wl.f)
+        V.vmc_set_walkers(h, occ)
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        V.vmc_sample(h, 1, 7)
+        V.vmc_measure(h, occ)
+        V.vmc_logpsi_backward(h)
+        torch.cuda.synchronize()
+        after = torch.cuda.mem_get_info()[0]
+        h.close()
+        return before, after
+
+    free_before_and_after()   # loads the kernels
+    before, after = free_before_and_after()
+    assert after == before
+
+
+def test_sample_sets_beyond_the_inverses_workspace():
+    """1.1 million samples of 16 electrons in FP64 hold more inverses than the workspace: they
+    go in pieces, with the samples and energies of a handle that needs one."""
+    wl = problem(9, 8, 8, "pairs")
+    nw, spw, few = 550001, 2, 3000
+    base = inputs.draw_configs(np.random.default_rng(1), 81, 9, 8, 8)
+    occ = np.ascontiguousarray(base[np.arange(nw) % len(base)])
+    h = V.vmc_create(wl, n_walkers=nw, samples_per_walker=spw)
+    g = V.vmc_create(wl, n_walkers=few, samples_per_walker=spw)
+    for x, o in ((h, occ), (g, occ[:few])):
+        V.vmc_set_params(x, wl.C, wl.f)
+        V.vmc_set_walkers(x, o)
+        V.vmc_sample(x, 1, 77)
+    so, sE, _, _ = V.vmc_get_samples(h)
+    go, gE, _, _ = V.vmc_get_samples(g)
+    assert np.array_equal(so[:few * spw], go) and np.array_equal(sE[:few * spw], gE)
+    # a configuration's energy does not depend on where it is evaluated
+    pick = np.random.default_rng(2).integers(0, nw * spw, few * spw)
+    V.vmc_measure(h, so)
+    mE = V.vmc_get_samples(h)[1]
+    V.vmc_measure(g, np.ascontiguousarray(so[pick]))
+    assert np.array_equal(V.vmc_get_samples(g)[1], mE[pick])
+    # nor on the chain, but for the drift of its rank-2 updates (1e-16 per update, times the
+    # condition of the blocks on the way); another sample's energy would be off by order one
+    assert np.mean(np.abs(sE[pick] - mE[pick]) <= 1e-6 * np.maximum(1.0, np.abs(mE[pick]))) >= 0.99
+    h.close()
+    g.close()
