@@ -258,8 +258,8 @@ __device__ void ab_same_spin(const DevProblem& pb, R* gss, const uint32_t* cidx,
 
 // sum over the occupied k of (pq|kk) - d(spin) (pk|kq), leaving out the
 // electron itself (orbital `own` of the given spin): the two-electron part of
-// the matrix element of a single move p -> q, and (p = q) of the diagonal.  The
-// integrals of one (p, q) are two consecutive rows.
+// the matrix element of a single move p -> q.  The integrals of one (p, q) are two
+// consecutive rows.
 template <typename R>
 __device__ __forceinline__ R coulomb_exchange(const DevProblem& pb, int p, int q, int own, uint64_t same, uint64_t other) {
     const int nk = pb.eri_nk;
@@ -572,11 +572,27 @@ __global__ void __launch_bounds__(kAbThreads, sizeof(R) == 4 ? 5 : 3) k_ab_energ
             }
         }
         double e = 0.0;
-        // diagonal: sum_k h_kk + 1/2 sum_{k != l} [(kk|ll) - d(s_k, s_l) (kl|lk)]
+        // diagonal: sum_k h_kk + sum_{k < l} [(kk|ll) - d(s_k, s_l) (kl|lk)], the largest
+        // part of E_L, in FP64
         for (int t = tid; t < N; t += bd) {
-            const bool d = occ[t] >= ns;
-            const int k = d ? occ[t] - ns : occ[t];
-            e += (double)load_h<R>(pb, k, k) + 0.5 * (double)coulomb_exchange<R>(pb, k, k, k, d ? dn : up, d ? up : dn);
+            const int k = occ[t] >= ns ? occ[t] - ns : occ[t];
+            e += (double)load_h<R>(pb, k, k);
+        }
+        {
+            const R* jk = sizeof(R) == 4 ? (const R*)pb.erijk32 : (const R*)pb.erijk64;
+            int l = 1, k = tid;
+            for (int t = tid; t < N * (N - 1) / 2; t += bd) {
+                while (k >= l) {
+                    k -= l;
+                    ++l;
+                }
+                const int ok = occ[k], ol = occ[l], sk = ok >= ns ? ok - ns : ok, sl = ol >= ns ? ol - ns : ol;
+                const R* J = jk + (size_t)(sk * ns + sk) * 2 * pb.eri_nk + sl;
+                R w = J[0];
+                if ((ok >= ns) == (ol >= ns)) w -= J[pb.eri_nk];
+                e += (double)w;
+                k += bd;
+            }
         }
         term_sum<R> sum;
         if (a.pairs) {

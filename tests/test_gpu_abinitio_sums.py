@@ -1,5 +1,6 @@
 """The ab initio local energy where a short cut would show: more electrons than a warp
-has lanes, samples that no walker wrote, sample sets larger than the workspace.
+has lanes, samples that no walker wrote, sample sets larger than the workspace,
+sums that FP32 cannot hold.
 """
 import numpy as np
 import pytest
@@ -104,3 +105,38 @@ def test_sample_sets_beyond_the_inverses_workspace():
     assert np.mean(np.abs(sE[pick] - mE[pick]) <= 1e-6 * np.maximum(1.0, np.abs(mE[pick]))) >= 0.99
     h.close()
     g.close()
+
+
+def singlet(n, phi, chol, h=None, corr_sites=(), C=None):
+    """Pairing f between up orbital i and down orbital j = phi[i, j] only."""
+    M = 2 * n
+    F = np.zeros((M, M))
+    F[:n, n:] = phi
+    sites = [np.asarray(s, np.int32) for s in corr_sites]
+    return inputs.Workload(name="s", n_sites=n, n_up=1, n_dn=1, ham=inputs.ABINITIO, corr_sites=sites,
+                           C=np.zeros(0) if C is None else C, f=F[np.triu_indices(M, 1)],
+                           h=np.zeros((n, n)) if h is None else h, chol=chol, n_walkers=1)
+
+
+@pytest.mark.parametrize("prec", [V.VMC_FP32, V.VMC_FP64])
+def test_diagonal_is_summed_beyond_fp32(prec):
+    """Diagonal factors L^mu: E_L is <n|H|n> alone, (kk|ll) odd integers below 2^22 (exact
+    in FP32) whose sum over pairs passes 2^24.  FP64 sums are exact."""
+    n, ne = 12, 6
+    rng = np.random.default_rng(5)
+    l = 2.0 * rng.integers(512, 1024, n) + 1.0
+    hd = rng.integers(1, 1 << 20, n).astype(np.float64)
+    phi = rng.standard_normal((n, n))
+    wl = singlet(n, phi, np.diag(l)[None], np.diag(hd))
+    wl.n_up = wl.n_dn = ne
+    cfgs = inputs.draw_configs(rng, 20, n, ne, ne)
+    want = []
+    for o in cfgs.astype(np.int64):
+        s = o % n
+        w = np.outer(l[s], l[s])   # (kk|ll); the exchange (kl|lk), k != l of one spin, vanishes
+        same = (o[:, None] >= n) == (o[None, :] >= n)
+        w[same & (s[:, None] == s[None, :])] = 0.0
+        want.append(hd[s].sum() + 0.5 * w.sum())
+    want = np.array(want)
+    assert want.max() > 2.0 ** 24
+    assert np.array_equal(energies(wl, cfgs, prec, prec == V.VMC_FP64, prec == V.VMC_FP32), want)
