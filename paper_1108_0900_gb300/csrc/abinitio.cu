@@ -352,7 +352,7 @@ __device__ __forceinline__ void ab_doubles_mixed(const DevProblem& pb, const AbL
                 const R* row = eri_table<R>(pb) + (i1 * ns + jx) * ns * ns;
 #pragma unroll
                 for (int u = 0; u < kAbSlots; ++u) hm[u] = __ldg(row + col[u]);
-                const R gxa = G[x * GS + a], fxa = load_F<R>(pb, jx, i1), omr = R(1) - gxa;
+                const R gxa = G[x * GS + a], fxa = load_F<R>(pb, jx, i1), omr = R(1) - gxa, rs = s1[a * eu + x];
                 __syncwarp();   // the last first move's vectors are read
 #pragma unroll
                 for (int w = 0; w < W; ++w) {
@@ -369,13 +369,12 @@ __device__ __forceinline__ void ab_doubles_mixed(const DevProblem& pb, const AbL
                         Quad<R> q;
                         q.x = el[w] ? v : fyx;
                         q.y = fma(el[w] ? fxa : -gxa, ua[w], el[w] ? -v : v);
-                        q.z = r;
+                        q.z = el[w] ? r * rs : r;   // with electron b: the first move's own factor
                         q.w = int_word(r, code);
                         ev[dst[w]] = q;
                     }
                 }
                 __syncwarp();
-                R part = R(0);
 #pragma unroll
                 for (int u = 0; u < kAbSlots; ++u) {
                     const Quad<R> B = ev[sb[u]], Y = ev[nd + sy[u]];
@@ -383,9 +382,8 @@ __device__ __forceinline__ void ab_doubles_mixed(const DevProblem& pb, const AbL
                     const R sv = fma(Y.x, omr, fma(fxa, c3[u], -fma(-fyb[u], B.x, Y.y)));
                     const R rpf = fma(-sv, xba[u], fma(gxa, t1, c2[u] * B.y));
                     const int t = c0 + 32 * u + lane;
-                    if (t < nd * ed) part = fma(hm[u] * rpf, B.z * Y.z * t2[4 * t + word_int(B.w) + word_int(Y.w)], part);
+                    if (t < nd * ed) sum.add(hm[u] * rpf * (B.z * Y.z * t2[4 * t + word_int(B.w) + word_int(Y.w)]));
                 }
-                sum.add(part * s1[a * eu + x]);
             }
         }
     }
@@ -455,14 +453,12 @@ __device__ __forceinline__ void ab_doubles_same(const DevProblem& pb, const AbLa
                 er[k] = rt[rs * s] * gss[i1 * ns + s] * gss[i2 * ns + s];
             }
             __syncwarp();
-            R part = R(0);
 #pragma unroll
             for (int u = 0; u < kAbPairSlots; ++u) {
                 const Quad<R> Vx = ev[sx[u]], Vy = ev[sy[u]];
                 const R rpf = double_ratio<R>(Vx.x, Vx.y, Vy.x, Vy.y, xab, xba, Vy.z, Vy.w, fyx[u], Vx.z, h[u]);
-                part = fma((hm[u] - hx[u]) * rpf, er[sx[u]] * er[sy[u]] * gxy[u], part);
+                sum.add((hm[u] - hx[u]) * rpf * (er[sx[u]] * er[sy[u]] * gxy[u] * rab));
             }
-            sum.add(part * rab);
             b += nw;
             while (b >= na && a < na) {
                 b = b - na + a + 2;

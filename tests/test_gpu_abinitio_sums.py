@@ -2,6 +2,8 @@
 has lanes, samples that no walker wrote, sample sets larger than the workspace,
 sums that FP32 cannot hold.
 """
+import itertools
+
 import numpy as np
 import pytest
 
@@ -140,3 +142,43 @@ def test_diagonal_is_summed_beyond_fp32(prec):
     want = np.array(want)
     assert want.max() > 2.0 ** 24
     assert np.array_equal(energies(wl, cfgs, prec, prec == V.VMC_FP64, prec == V.VMC_FP32), want)
+
+
+@pytest.mark.parametrize("prec", [V.VMC_FP32, V.VMC_FP64])
+def test_every_double_excitation_enters_the_wide_sum(prec):
+    """Factors between occupied and empty orbitals only: E_L is the double excitations
+    alone.  Integrals (small odd numbers times powers of two, one of the two of a
+    same-spin move zero or both equal) and amplitude ratios (integers, by an identity
+    pairing of the occupied block) make every term exact in FP32; a sum in FP32
+    rounds, one in FP32 pairs keeps 48 bits."""
+    n, ne = 26, 6
+    rng = np.random.default_rng(11)
+    O, X = np.arange(ne), np.arange(ne, n)
+    phi = rng.integers(-1, 2, (n, n))
+    phi[np.ix_(O, O)] = np.eye(ne)
+    u = (2 * rng.integers(0, 4, n) + 1) * 2 ** np.where(np.arange(n) < ne, 0, rng.choice([0, 14], n)) * rng.choice([-1, 1], n)
+    L = np.zeros((1, n, n))
+    L[0][:3, 6:16] = np.outer(u[:3], u[6:16])
+    L[0][3:6, 16:] = np.outer(u[3:6], u[16:])
+    L[0] += L[0].T
+    wl = singlet(n, phi.astype(np.float64), L)
+    wl.n_up = wl.n_dn = ne
+    cfg = np.concatenate([O, O + n]).astype(np.uint8)[None]
+    Li = L[0].astype(np.int64)
+
+    def ratio(rows, cols):
+        return int(np.rint(np.linalg.det(phi[np.ix_(rows, cols)].astype(np.float64))))
+
+    terms = []
+    for a, x in itertools.product(O, X):          # up a -> x, down b -> y
+        rows = np.where(O == a, x, O)
+        terms += [int(Li[a, x] * Li[b, y]) * ratio(rows, np.where(O == b, y, O)) for b, y in itertools.product(O, X)]
+    for a, b in itertools.combinations(O, 2):     # two of one spin
+        for x, y in itertools.combinations(X, 2):
+            to = np.where(O == a, x, np.where(O == b, y, O))
+            m = int(Li[a, x] * Li[b, y] - Li[a, y] * Li[b, x])
+            terms += [m * ratio(to, O), m * ratio(O, to)]
+    assert all(t == int(np.float32(t)) for t in terms)
+    E = energies(wl, cfg, prec, prec == V.VMC_FP64, prec == V.VMC_FP32)
+    # about 100 additions per lane, each good to 2^-48 of the lane's sum of magnitudes
+    assert abs(E[0] - sum(terms)) <= 2.0 ** -40 * sum(map(abs, terms))
