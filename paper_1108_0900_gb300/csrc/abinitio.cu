@@ -313,7 +313,7 @@ __device__ __forceinline__ void ab_doubles_mixed(const DevProblem& pb, const AbL
     const int xm = (eu + 1) / 2;   // a warp's unit of work: one a, half of the x
     for (int c0 = 0; c0 < nd * ed; c0 += 32 * kAbSlots) {
         // the lane's second moves (b, y): the integral column, G[y][b], F[y][o_b];
-        // slots past the end weigh zero
+        // slots past the end read an integral of zero
         int sb[kAbSlots], sy[kAbSlots], col[kAbSlots];
         R gyb[kAbSlots], fyb[kAbSlots];
 #pragma unroll
@@ -351,7 +351,7 @@ __device__ __forceinline__ void ab_doubles_mixed(const DevProblem& pb, const AbL
                 const int jx = emp[x];
                 const R* row = eri_table<R>(pb) + (i1 * ns + jx) * ns * ns;
 #pragma unroll
-                for (int u = 0; u < kAbSlots; ++u) hm[u] = __ldg(row + col[u]);
+                for (int u = 0; u < kAbSlots; ++u) hm[u] = c0 + 32 * u + lane < nd * ed ? __ldg(row + col[u]) : R(0);
                 const R gxa = G[x * GS + a], fxa = load_F<R>(pb, jx, i1), omr = R(1) - gxa, rs = s1[a * eu + x];
                 __syncwarp();   // the last first move's vectors are read
 #pragma unroll
@@ -381,8 +381,9 @@ __device__ __forceinline__ void ab_doubles_mixed(const DevProblem& pb, const AbL
                     const R t1 = fma(Y.x, xab[u], c1[u]);
                     const R sv = fma(Y.x, omr, fma(fxa, c3[u], -fma(-fyb[u], B.x, Y.y)));
                     const R rpf = fma(-sv, xba[u], fma(gxa, t1, c2[u] * B.y));
-                    const int t = c0 + 32 * u + lane;
-                    if (t < nd * ed) sum.add(hm[u] * rpf * (B.z * Y.z * t2[4 * t + word_int(B.w) + word_int(Y.w)]));
+                    const int t = min(c0 + 32 * u + lane, nd * ed - 1);
+                    const R term = hm[u] * rpf * (B.z * Y.z * t2[4 * t + word_int(B.w) + word_int(Y.w)]);
+                    sum.add(hm[u] == R(0) ? R(0) : term);   // a vanishing integral's ratio may overflow
                 }
             }
         }
@@ -457,7 +458,9 @@ __device__ __forceinline__ void ab_doubles_same(const DevProblem& pb, const AbLa
             for (int u = 0; u < kAbPairSlots; ++u) {
                 const Quad<R> Vx = ev[sx[u]], Vy = ev[sy[u]];
                 const R rpf = double_ratio<R>(Vx.x, Vx.y, Vy.x, Vy.y, xab, xba, Vy.z, Vy.w, fyx[u], Vx.z, h[u]);
-                sum.add((hm[u] - hx[u]) * rpf * (er[sx[u]] * er[sy[u]] * gxy[u] * rab));
+                const R d = hm[u] - hx[u];
+                const R term = d * rpf * (er[sx[u]] * er[sy[u]] * gxy[u] * rab);
+                sum.add(d == R(0) ? R(0) : term);
             }
             b += nw;
             while (b >= na && a < na) {

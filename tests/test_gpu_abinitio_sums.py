@@ -1,6 +1,6 @@
 """The ab initio local energy where a short cut would show: more electrons than a warp
 has lanes, samples that no walker wrote, sample sets larger than the workspace,
-sums that FP32 cannot hold.
+sums that FP32 cannot hold, integrals of zero beside ratios that overflow.
 """
 import itertools
 
@@ -182,3 +182,23 @@ def test_every_double_excitation_enters_the_wide_sum(prec):
     E = energies(wl, cfg, prec, prec == V.VMC_FP64, prec == V.VMC_FP32)
     # about 100 additions per lane, each good to 2^-48 of the lane's sum of magnitudes
     assert abs(E[0] - sum(terms)) <= 2.0 ** -40 * sum(map(abs, terms))
+
+
+@pytest.mark.parametrize("prec,big", [(V.VMC_FP32, 1e25), (V.VMC_FP64, 1e200)])
+def test_vanishing_integrals_meet_no_ratio(prec, big):
+    """Pairing amplitudes of the empty orbitals so large that the ratios of double moves
+    overflow: with integrals of zero these moves do not enter E_L."""
+    n, ne = 8, 4
+    rng = np.random.default_rng(9)
+    O, X = np.arange(ne), np.arange(ne, n)
+    phi = rng.standard_normal((n, n))
+    phi[X] *= big
+    phi[np.ix_(O, X)] *= big
+    hd = rng.integers(1, 100, n).astype(np.float64)
+    l = 1.0 + np.arange(n)
+    wl = singlet(n, phi, np.diag(l)[None], np.diag(hd))
+    wl.n_up = wl.n_dn = ne
+    cfg = np.concatenate([O, O + n]).astype(np.uint8)[None]
+    w = np.outer(l[O], l[O])
+    want = 2.0 * hd[O].sum() + 0.5 * (4.0 * w.sum() - 2.0 * np.trace(w))   # no self interaction
+    assert energies(wl, cfg, prec, prec == V.VMC_FP64, prec == V.VMC_FP32)[0] == want
