@@ -113,6 +113,75 @@ __device__ __forceinline__ int site_state(uint64_t up, uint64_t dn, int s) {
     return (int)((up >> s) & 1ull) + 2 * (int)((dn >> s) & 1ull);
 }
 
+// Factors of the sites' local states: rsite[4 s + v] = product over the correlators
+// on site s of C(s in state v) / C(now), all other sites as they are.
+template <typename R>
+__device__ __forceinline__ void site_factors(const DevProblem& pb, R* rsite, const uint32_t* cidx, uint64_t up, uint64_t dn) {
+    for (int t = threadIdx.x; t < 4 * pb.ns; t += blockDim.x) {
+        const int s = t >> 2, v = t & 3, n = site_state(up, dn, s);
+        R f = R(1);
+        if (v != n)
+            for (int ent = pb.site_cptr[s]; ent < pb.site_cptr[s + 1]; ++ent) {
+                const int c = pb.site_corr[ent];
+                const int64_t k = pb.corr_off[c] + (int64_t)cidx[c];
+                f *= load_C<R>(pb, k + pb.site_w[ent] * (v - n)) / load_C<R>(pb, k);
+            }
+        rsite[t] = f;
+    }
+}
+
+// Correlator factor, for correlators of at most two sites, of a move that changes
+// the local state of site S[k] by D[k], k < n (repeated sites add up): the sites'
+// factors, and per correlator on two of them C(both) C(now) / (C(one) C(other)).
+// Only states before and after the move enter.
+template <typename R, int n>
+__device__ R site_move_factor(const DevProblem& pb, const uint32_t* cidx, const R* rsite, uint64_t up, uint64_t dn,
+                              int (&S)[n], int (&D)[n]) {
+#pragma unroll
+    for (int k = 1; k < n; ++k)
+#pragma unroll
+        for (int m = 0; m < k; ++m)
+            if (S[k] == S[m]) {
+                D[m] += D[k];
+                D[k] = 0;   // (a later equal site adds to the first of its kind)
+                break;
+            }
+    R f = R(1);
+#pragma unroll
+    for (int k = 0; k < n; ++k)
+        if (D[k] != 0) f *= rsite[4 * S[k] + site_state(up, dn, S[k]) + D[k]];
+#pragma unroll
+    for (int k = 0; k < n; ++k)
+#pragma unroll
+        for (int m = k + 1; m < n; ++m) {
+            if (D[k] == 0 || D[m] == 0) continue;
+            const int st = S[k] * pb.ns + S[m];
+            for (int e = pb.pair_ptr[st]; e < pb.pair_ptr[st + 1]; ++e) {
+                const int c = pb.pair_corr[e];
+                const int64_t o = pb.corr_off[c] + (int64_t)cidx[c];
+                const int dk = site_weight_in(pb, c, S[k]) * D[k], dm = site_weight_in(pb, c, S[m]) * D[m];
+                f *= load_C<R>(pb, o + dk + dm) * load_C<R>(pb, o) / (load_C<R>(pb, o + dk) * load_C<R>(pb, o + dm));
+            }
+        }
+    return f;
+}
+
+// Magnitudes that the tables of ab_tables may hold: with toggle factors within
+// 2^+-kToggle and corrections within 2^+-kCorrection the product of an excitation,
+// at most four of the former and six of the latter, stays a normal number at
+// every step.  An excitation of moderate factor may pass through toggles that are
+// not (two electrons of a site moved together where single occupancy is
+// projected out), so a sample beyond goes the general way.
+template <typename R> struct TableRange;
+template <> struct TableRange<float> { static constexpr int kToggle = 20, kCorrection = 7; };      // 122 of 126
+template <> struct TableRange<double> { static constexpr int kToggle = 200, kCorrection = 30; };   // 980 of 1022
+__device__ __forceinline__ bool beyond(float v, int lim) {   // zero, infinite and NaN too
+    return (uint32_t)(((__float_as_int(v) >> 23) & 255) - (127 - lim)) > 2u * (uint32_t)lim;
+}
+__device__ __forceinline__ bool beyond(double v, int lim) {
+    return (uint32_t)(((__double2hiint(v) >> 20) & 0x7ff) - (1023 - lim)) > 2u * (uint32_t)lim;
+}
+
 template <typename R> __device__ __forceinline__ const R* eri_table(const DevProblem& pb);
 template <> __device__ __forceinline__ const float* eri_table<float>(const DevProblem& pb) { return pb.eri32; }
 template <> __device__ __forceinline__ const double* eri_table<double>(const DevProblem& pb) { return pb.eri64; }
@@ -171,29 +240,27 @@ __device__ __forceinline__ void for_site_pairs(int ns, F f) {
     }
 }
 
+// Returns whether an entry of the thread's is beyond TableRange.
 template <typename R>
-__device__ void ab_tables(const DevProblem& pb, const AbLayout& L, R* tab, const uint32_t* cidx,
+__device__ bool ab_tables(const DevProblem& pb, const AbLayout& L, R* tab, const uint32_t* cidx,
                           const int8_t* orb_pos, const int8_t* eidx, uint64_t up, uint64_t dn) {
+    constexpr int kT = TableRange<R>::kToggle, kC = TableRange<R>::kCorrection;
+    bool out = false;
     const int ns = pb.ns, nu = pb.nu, eu = ns - nu, ed = ns - pb.nd;
     R *rup = tab + L.rup, *rdn = tab + L.rdn, *g0 = tab + L.g0, *g1 = tab + L.g1, *t2 = tab + L.t2;
     R* rsite = t2;   // the factors of site s in every local state, until t2 is built
-    for (int t = threadIdx.x; t < 4 * ns; t += blockDim.x) {
-        const int s = t >> 2, v = t & 3, n = site_state(up, dn, s);
-        R f = R(1);
-        if (v != n)
-            for (int ent = pb.site_cptr[s]; ent < pb.site_cptr[s + 1]; ++ent) {
-                const int c = pb.site_corr[ent];
-                const int64_t k = pb.corr_off[c] + (int64_t)cidx[c];
-                f *= load_C<R>(pb, k + pb.site_w[ent] * (v - n)) / load_C<R>(pb, k);
-            }
-        rsite[t] = f;
-    }
+    site_factors<R>(pb, rsite, cidx, up, dn);
     for (int s = threadIdx.x; s < ns; s += blockDim.x) g0[s * ns + s] = R(1);
     __syncthreads();
     for (int t = threadIdx.x; t < 2 * ns; t += blockDim.x) {
         const int s = t >> 1, n = site_state(up, dn, s) ^ (t & 1);
-        rdn[t] = rsite[4 * s + (n ^ 2)] / rsite[4 * s + n];
-        if (t & 1) rup[s] = rsite[4 * s + n];
+        const R f = rsite[4 * s + (n ^ 2)] / rsite[4 * s + n];
+        rdn[t] = f;
+        out |= beyond(f, kT);
+        if (t & 1) {
+            rup[s] = rsite[4 * s + n];
+            out |= beyond(rsite[4 * s + n], kT);
+        }
     }
     __syncthreads();
     for_site_pairs(ns, [&](int s, int t) {
@@ -220,15 +287,18 @@ __device__ void ab_tables(const DevProblem& pb, const AbLayout& L, R* tab, const
         }
         g0[t * ns + s] = a0;
         g0[s * ns + t] = b0;
+        out |= beyond(a0, kC) | beyond(b0, kC);
         const bool us = vs & 1, ut = vt & 1, ds = vs & 2, dt = vt & 2;
         if (us != ut) {
             const int a = orb_pos[us ? s : t], x = eidx[us ? t : s];
+            out |= beyond(a1, kC) | beyond(b1, kC);
             g1[a * eu + x] = us ? a1 * rdn[2 * s + 1] : b1 * rdn[2 * t + 1];
             g1[nu * eu + x * nu + a] = us ? b1 * rdn[2 * t + 1] : a1 * rdn[2 * s + 1];
         }
         if (ds != dt) {
             const int b = orb_pos[(ds ? s : t) + ns] - nu, y = eidx[(ds ? t : s) + ns] - eu;
             R* q = t2 + 4 * (b * ed + y);
+            out |= beyond(d[0], kC) | beyond(d[1], kC) | beyond(d[2], kC) | beyond(d[3], kC);
             q[0] = d[0];
             q[1] = ds ? d[1] : d[2];
             q[2] = ds ? d[2] : d[1];
@@ -236,11 +306,14 @@ __device__ void ab_tables(const DevProblem& pb, const AbLayout& L, R* tab, const
         }
     });
     __syncthreads();
+    return out;
 }
 
+// (the caller synchronises)
 template <typename R>
-__device__ void ab_same_spin(const DevProblem& pb, R* gss, const uint32_t* cidx, uint64_t up, uint64_t dn, int spin) {
+__device__ bool ab_same_spin(const DevProblem& pb, R* gss, const uint32_t* cidx, uint64_t up, uint64_t dn, int spin) {
     const int ns = pb.ns, m = spin + 1;
+    bool out = false;
     for (int s = threadIdx.x; s < ns; s += blockDim.x) gss[s * ns + s] = R(0);
     for_site_pairs(ns, [&](int s, int t) {
         R g = R(1);
@@ -252,8 +325,9 @@ __device__ void ab_same_spin(const DevProblem& pb, R* gss, const uint32_t* cidx,
             g *= load_C<R>(pb, k + ds + dt) * load_C<R>(pb, k) / (load_C<R>(pb, k + ds) * load_C<R>(pb, k + dt));
         }
         gss[s * ns + t] = gss[t * ns + s] = g;
+        out |= beyond(g, TableRange<R>::kCorrection);
     });
-    __syncthreads();
+    return out;
 }
 
 // sum over the occupied k of (pq|kk) - d(spin) (pk|kq), leaving out the
@@ -488,7 +562,7 @@ __global__ void __launch_bounds__(kAbThreads, sizeof(R) == 4 ? 5 : 3) k_ab_energ
     uint8_t* emp = occ + 64;
     int8_t* orb_pos = (int8_t*)(emp + 128);
     int8_t* eidx = orb_pos + 128;
-    R *G = tab + L.G, *Rs = tab + L.g0;          // Rs: the general path's single-move factors
+    R *G = tab + L.G, *Rs = tab + L.g0;          // Rs: the general path's single-move or site factors
     const uint64_t smask = (ns == 64) ? ~0ull : ((1ull << ns) - 1ull);
 
     for (int64_t s = blockIdx.x; s < a.n_s; s += gridDim.x) {
@@ -551,7 +625,8 @@ __global__ void __launch_bounds__(kAbThreads, sizeof(R) == 4 ? 5 : 3) k_ab_energ
                     if (W > 1 && lane + 32 < N) G[(h0 + u) * GS + lane + 32] = acc[u][1];
                 }
         }
-        if (a.pairs) ab_tables<R>(pb, L, tab, cidx, orb_pos, eidx, up, dn);
+        bool out = false;   // a table's entry of this thread is beyond the range
+        if (a.pairs) out = ab_tables<R>(pb, L, tab, cidx, orb_pos, eidx, up, dn);
         __syncthreads();
         // H over pairs of empty orbitals y > x, by class [x][y]
         {
@@ -594,19 +669,23 @@ __global__ void __launch_bounds__(kAbThreads, sizeof(R) == 4 ? 5 : 3) k_ab_energ
             }
         }
         term_sum<R> sum;
+        double e1 = 0.0;         // singles
+        bool general = !a.pairs;
         if (a.pairs) {
             R *rup = tab + L.rup, *rdn = tab + L.rdn, *gss = tab + L.gss, *s1 = tab + L.s1;
             for (int sp = 0; sp < 2; ++sp) {
                 const int a0 = sp ? nu : 0, na = sp ? nd : nu, x0 = sp ? eu : 0, nx = sp ? ed : eu, o1 = sp ? ns : 0;
                 __syncthreads();
-                ab_same_spin<R>(pb, gss, cidx, up, dn, sp);
+                out |= ab_same_spin<R>(pb, gss, cidx, up, dn, sp);
+                general = __syncthreads_or(out);
+                if (general) break;
                 // singles, and their correlator factors s1[a][x]
                 for (int t = tid; t < na * nx; t += bd) {
                     const int ia = a0 + t / nx, ix = x0 + t % nx, p = occ[ia], q = emp[ix], sp_ = p - o1, sq = q - o1;
                     const R r = (sp ? rdn[2 * sp_] * rdn[2 * sq] : rup[sp_] * rup[sq]) * gss[sp_ * ns + sq];
                     s1[t] = r;
                     const R hm = load_h<R>(pb, sp_, sq) + coulomb_exchange<R>(pb, sp_, sq, sp_, sp ? dn : up, sp ? up : dn);
-                    e += (double)(hm * G[ix * GS + ia] * r);
+                    e1 += (double)(hm * G[ix * GS + ia] * r);
                 }
                 __syncthreads();
                 ab_doubles_same<R>(pb, L, tab, X, XS, occ, emp, sp, sum);
@@ -615,12 +694,20 @@ __global__ void __launch_bounds__(kAbThreads, sizeof(R) == 4 ? 5 : 3) k_ab_energ
                     ab_doubles_mixed<R, W>(pb, L, tab, X, XS, occ, orb_pos, emp, eidx, dn, sum);
                 }
             }
-        } else {
-            // single-move correlator factors Rs[a][ie] (same spin only)
-            for (int t = tid; t < N * E; t += bd) {
-                const int p = occ[t / E], q = emp[t % E];
-                Rs[t] = ((p >= ns) == (q >= ns)) ? corr_ratio_serial<R>(pb, cidx, p, q) : R(0);
-            }
+        }
+        if (general) {
+            // correlators of more sites, tables that do not fit or do not hold: every
+            // excitation's factor by itself, from the sites' factors or (more sites)
+            // those of the single moves, Rs[a][ie] (same spin only)
+            const bool sites2 = pb.max_csites <= 2;
+            sum = term_sum<R>();
+            e1 = 0.0;
+            if (sites2) site_factors<R>(pb, Rs, cidx, up, dn);
+            else
+                for (int t = tid; t < N * E; t += bd) {
+                    const int p = occ[t / E], q = emp[t % E];
+                    Rs[t] = ((p >= ns) == (q >= ns)) ? corr_ratio_serial<R>(pb, cidx, p, q) : R(0);
+                }
             __syncthreads();
             for (int t = tid; t < N * E; t += bd) {
                 const int ia = t / E, ie = t % E;
@@ -629,7 +716,12 @@ __global__ void __launch_bounds__(kAbThreads, sizeof(R) == 4 ? 5 : 3) k_ab_energ
                 const bool d = p >= ns;
                 const int ip = d ? p - ns : p, iq = d ? x - ns : x;
                 const R hm = load_h<R>(pb, ip, iq) + coulomb_exchange<R>(pb, ip, iq, ip, d ? dn : up, d ? up : dn);
-                e += (double)(hm * G[ie * GS + ia] * Rs[t]);
+                R r;
+                if (sites2) {
+                    int S[2] = {ip, iq}, D[2] = {d ? -2 : -1, d ? 2 : 1};
+                    r = site_move_factor<R, 2>(pb, cidx, Rs, up, dn, S, D);
+                } else r = Rs[t];
+                e1 += (double)(hm * G[ie * GS + ia] * r);
             }
             // doubles: up-up, down-down and up-down classes.  Within a class the
             // threads run over (electron pair, empty pair) with the electron pair
@@ -665,12 +757,17 @@ __global__ void __launch_bounds__(kAbThreads, sizeof(R) == 4 ? 5 : 3) k_ab_energ
                     const R rpf = double_ratio<R>(G[ix * GS + ia], G[ix * GS + ib], G[iy * GS + ia], G[iy * GS + ib],
                                                   X[ia * XS + ib], X[ib * XS + ia], load_F<R>(pb, y, p1),
                                                   load_F<R>(pb, y, p2), load_F<R>(pb, y, x), load_F<R>(pb, x, p1), h);
-                    sum.add(hm * rpf *
-                            corr_ratio_double<R>(pb, cidx, p1, x, p2, y, Rs[ia * E + ix], Rs[ib * E + iy]));
+                    R r;
+                    if (sites2) {
+                        const int f1 = p1 >= ns ? 2 : 1, f2 = p2 >= ns ? 2 : 1;
+                        int S[4] = {p1 % ns, x % ns, p2 % ns, y % ns}, D[4] = {-f1, f1, -f2, f2};
+                        r = site_move_factor<R, 4>(pb, cidx, Rs, up, dn, S, D);
+                    } else r = corr_ratio_double<R>(pb, cidx, p1, x, p2, y, Rs[ia * E + ix], Rs[ib * E + iy]);
+                    sum.add(hm * rpf * r);
                 }
             }
         }
-        e = warp_sum(e + sum.value());
+        e = warp_sum(e + e1 + sum.value());
         if (lane == 0) red[wid] = e;
         __syncthreads();
         if (tid == 0) {

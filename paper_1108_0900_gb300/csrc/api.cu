@@ -924,7 +924,7 @@ static int ab_energy(vmc_ctx* h, bool fp64, int64_t s0, int64_t n_s, cudaStream_
         nw = kAbThreads / 32;
         L = ab_layout(h->ns, h->nu, h->nd, nw);
     }
-    a.elems = (int)round_up(a.pairs ? L.n : L.g0 + h->N * (h->M - h->N), 4);
+    a.elems = (int)round_up(a.pairs ? L.n : L.g0 + std::max(h->N * (h->M - h->N), 4 * h->ns), 4);
     const size_t smem = a.elems * rsz + rest;
     if (smem + 64 > h->smem_optin) return VMC_ERR_UNSUPPORTED;
     VCK(launch_ab_energy(fp64, a, 32 * nw, smem, h->nsm, st));

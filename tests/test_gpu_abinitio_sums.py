@@ -1,6 +1,7 @@
 """The ab initio local energy where a short cut would show: more electrons than a warp
 has lanes, samples that no walker wrote, sample sets larger than the workspace,
-sums that FP32 cannot hold, integrals of zero beside ratios that overflow.
+sums that FP32 cannot hold, integrals of zero beside ratios that overflow,
+correlators whose single toggles leave the walker's range.
 """
 import itertools
 
@@ -202,3 +203,28 @@ def test_vanishing_integrals_meet_no_ratio(prec, big):
     w = np.outer(l[O], l[O])
     want = 2.0 * hd[O].sum() + 0.5 * (4.0 * w.sum() - 2.0 * np.trace(w))   # no self interaction
     assert energies(wl, cfg, prec, prec == V.VMC_FP64, prec == V.VMC_FP32)[0] == want
+
+
+@pytest.mark.parametrize("prec,single", [(V.VMC_FP32, 1e-6), (V.VMC_FP32, 1e6), (V.VMC_FP64, 1e-40)])
+def test_correlators_that_project_single_occupancy(prec, single):
+    """Pair correlators that suppress (or favour) singly occupied sites by `single` each:
+    the 13 factors of one site together leave the precision's range, those of moving
+    a pair of electrons stay near one.  Tolerances as in test_gpu_abinitio_energy.py."""
+    n, ne = 14, 7
+    wl = problem(n, ne, ne, "pairs")
+    rng = np.random.default_rng(17)
+    u = np.array([1.0, single, single, 1.0]) if single < 1.0 else np.array([1.0 / single, 1.0, 1.0, 1.0 / single])
+    C = np.concatenate([np.outer(u, u).reshape(-1) for _ in wl.corr_sites])
+    wl.C = C * (1.0 + 0.05 * rng.uniform(-1.0, 1.0, len(C)))
+    up = inputs.draw_configs(rng, 4, n, ne, ne)[:, :ne]
+    if single < 1.0:
+        cfgs = np.concatenate([up, up + n], 1).astype(np.uint8)     # closed shells
+    else:
+        empty = np.array([[s for s in range(n) if s not in set(r)] for r in up])
+        cfgs = np.concatenate([up, empty + n], 1).astype(np.uint8)  # every site singly occupied
+    E_or = oracle.Problem(wl).measure(cfgs)[0]
+    assert np.all(np.isfinite(E_or))
+    kappa, scale = condition(wl, cfgs), np.maximum(1.0, np.abs(E_or))
+    eps = 1e-4 if prec == V.VMC_FP32 else 1e-12
+    E = energies(wl, cfgs, prec, prec == V.VMC_FP64, prec == V.VMC_FP32)
+    assert np.all(np.abs(E - E_or) <= eps * kappa * scale)
