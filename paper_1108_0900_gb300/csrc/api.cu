@@ -5,6 +5,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <set>
 #include <vector>
 
 #include "kernels.h"
@@ -49,14 +50,8 @@ struct vmc_ctx {
     int64_t ncap = 0, n_s = 0;
     int wprec = VMC_FP64, keep64 = 1, keeplow = 0, refresh_every = 0, fp64_refresh = 0;
     int ham = 0;
-    int maxd = 1, mind = 1 << 30;   // states of the largest and smallest correlator
-    std::vector<int> dims;          // and of every one
-    int mid_d(int most) const {     // of the largest with at most `most`
-        int d = 0;
-        for (int x : dims)
-            if (x <= most) d = std::max(d, x);
-        return d;
-    }
+    int maxd = 1;                // states of the largest correlator
+    std::set<std::pair<int, int>> unit_kinds;   // states and correlators of the histogram-scatter work units
     int max_csites = 0;          // sites of the largest correlator
     struct PassPlan {            // launch shape of a pass with FP64 sums (see plan_pass)
         int ni = 0;              // images per CTA
@@ -306,8 +301,6 @@ extern "C" int vmc_create(const vmc_lattice* lat, const vmc_hamiltonian* ham, co
         }
         cptr[c + 1] = (int)csites.size();
         h->maxd = std::max(h->maxd, 1 << (2 * m));
-        h->mind = std::min(h->mind, 1 << (2 * m));
-        h->dims.push_back(1 << (2 * m));
     }
     // classes: correlators of one class share one parameter block; blocks in
     // class order, corr_off[c] = first parameter of c's block
@@ -338,8 +331,10 @@ extern "C" int vmc_create(const vmc_lattice* lat, const vmc_hamiltonian* ham, co
     // histogram-scatter work units: up to kInstPerUnit correlators of one class
     std::vector<int4> units;
     for (int q = 0; q < h->n_class; ++q)
-        for (int j = class_ptr[q]; j < class_ptr[q + 1]; j += kInstPerUnit)
+        for (int j = class_ptr[q]; j < class_ptr[q + 1]; j += kInstPerUnit) {
             units.push_back(make_int4(q, j, std::min(j + kInstPerUnit, class_ptr[q + 1]), 0));
+            h->unit_kinds.insert({1 << (2 * cm[q]), units.back().z - j});
+        }
     h->n_units = (int)units.size();
     h->corr_off.assign(h->ncorr + 1, 0);
     for (int c = 0; c < h->ncorr; ++c) h->corr_off[c] = class_off[cls[c]];
@@ -1497,8 +1492,8 @@ static int launch_corr(vmc_ctx* h, const AT* T, const int* stop, cudaStream_t st
         VCK(cudaGetLastError());
         return VMC_OK;
     }
-    // a histogram per thread for classes of at most 64 values
-    if (h->mind * K <= 64) smem = std::max(smem, (size_t)h->mid_d(64 / K) * K * (256 + 1) * sizeof(AT));
+    for (const auto& [d, n] : h->unit_kinds)   // a histogram per thread
+        if (corr_columns(d, K, h->n_s * n)) smem = std::max(smem, (size_t)d * K * (256 + 1) * sizeof(AT));
     a.cap = (int)(smem / sizeof(AT));
     auto kern = k_corr_scatter<AT, K>;
     VCK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

@@ -20,8 +20,8 @@ namespace vmc {
 // samples per step (two 16-byte loads of states, K x 8 values of t).  Every
 // CTA of the cluster must call this.
 //
-// Classes of few states (4^m K values for every thread of the CTA within the
-// `cap` elements of h: up to 64 values at 256 threads): 32 lanes would meet on a
+// Classes of few states and many samples (corr_columns; 4^m K values for every
+// thread of the CTA within the `cap` elements of h): 32 lanes would meet on a
 // handful of addresses, and an FP64 shared atomic is a compare-and-swap loop.
 // Every thread then keeps a histogram of its own (column threadIdx.x, no
 // conflicts, no atomics), added up by warps before the cluster's sum.  Two-site
@@ -37,7 +37,7 @@ __device__ __forceinline__ void corr_cluster_histogram(const CorrArgs<AT>& a, AT
     const int q = unit.x;
     const int64_t off = pb.class_off[q];
     const int d = (int)(pb.class_off[q + 1] - off);
-    const bool own = (int64_t)d * K * (bd + 1) <= a.cap;
+    const bool own = corr_columns(d, K, a.n_s * (unit.z - unit.y)) && (int64_t)d * K * (bd + 1) <= a.cap;
     const int cols = own ? bd : 1;
     for (int i = threadIdx.x; i < d * K * cols; i += bd) h[i] = AT(0);
     __syncthreads();
