@@ -1492,8 +1492,14 @@ static int launch_corr(vmc_ctx* h, const AT* T, const int* stop, cudaStream_t st
         VCK(cudaGetLastError());
         return VMC_OK;
     }
-    for (const auto& [d, n] : h->unit_kinds)   // a histogram per thread
-        if (corr_columns(d, K, h->n_s * n)) smem = std::max(smem, (size_t)d * K * (256 + 1) * sizeof(AT));
+    // a histogram per thread
+    const double fu = (double)h->nu / h->ns, fd = (double)h->nd / h->ns;
+    const double agree = (fu * fu + (1 - fu) * (1 - fu)) * (fd * fd + (1 - fd) * (1 - fd));   // of one site
+    double eff = 1.0;
+    for (int m = 1; m < 4; ++m) a.from[m] = corr_columns_from(1 << (2 * m), eff /= agree, K);
+    for (const auto& [d, n] : h->unit_kinds)
+        if (d * K <= 64 && (double)h->n_s * n >= a.from[d == 4 ? 1 : d == 16 ? 2 : 3])
+            smem = std::max(smem, (size_t)d * K * (256 + 1) * sizeof(AT));
     a.cap = (int)(smem / sizeof(AT));
     auto kern = k_corr_scatter<AT, K>;
     VCK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

@@ -2,6 +2,7 @@
 // the stand-alone correlator kernel and the fused scatter kernel.
 #pragma once
 #include <cooperative_groups.h>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -20,7 +21,7 @@ namespace vmc {
 // samples per step (two 16-byte loads of states, K x 8 values of t).  Every
 // CTA of the cluster must call this.
 //
-// Classes of few states and many samples (corr_columns; 4^m K values for every
+// Classes of few states and many samples (corr_columns_from; 4^m K values for every
 // thread of the CTA within the `cap` elements of h): 32 lanes would meet on a
 // handful of addresses, and an FP64 shared atomic is a compare-and-swap loop.
 // Every thread then keeps a histogram of its own (column threadIdx.x, no
@@ -37,52 +38,57 @@ __device__ __forceinline__ void corr_cluster_histogram(const CorrArgs<AT>& a, AT
     const int q = unit.x;
     const int64_t off = pb.class_off[q];
     const int d = (int)(pb.class_off[q + 1] - off);
-    const bool own = corr_columns(d, K, a.n_s * (unit.z - unit.y)) && (int64_t)d * K * (bd + 1) <= a.cap;
+    const bool own = d * K <= 64 && (int64_t)d * K * (bd + 1) <= a.cap &&
+                     (double)a.n_s * (unit.z - unit.y) >= a.from[(31 - __clz(d)) / 2];
     const int cols = own ? bd : 1;
     for (int i = threadIdx.x; i < d * K * cols; i += bd) h[i] = AT(0);
     __syncthreads();
-    auto add = [&](int state, const AT* t) {
-#pragma unroll
-        for (int kk = 0; kk < K; ++kk) {
-            if (own) h[(state * K + kk) * bd + threadIdx.x] += t[kk];
-            else atomicAdd(&h[state * K + kk], t[kk]);
-        }
-    };
     const int64_t len = ((a.n_s + kCorrCluster - 1) / kCorrCluster + 7) & ~(int64_t)7;
     const int64_t s0 = min(a.n_s, rank * len), s1 = min(a.n_s, s0 + len);
     // 16-byte loads need the rows to start on a 16-byte boundary
     const bool vec = ((a.n_s & 7) == 0);
-    for (int ji = unit.y; ji < unit.z; ++ji) {
-        const cstate_t* st = a.cidxT + (int64_t)pb.class_inst[ji] * a.n_s;
-        int64_t s = s0;
-        if (vec) {
-            for (int64_t g = s0 + 8 * (int64_t)threadIdx.x; g + 8 <= s1; g += 8 * (int64_t)bd) {
-                const uint4 sa = *(const uint4*)(st + g), sb = *(const uint4*)(st + g + 4);
-                const uint32_t w8[8] = {sa.x, sa.y, sa.z, sa.w, sb.x, sb.y, sb.z, sb.w};
-                AT tv[8 * K];
+    auto run = [&](auto columns) {   // a loop of its own for either form
+        auto add = [&](int state, const AT* t) {
 #pragma unroll
-                for (int j = 0; j < 8 * K; ++j) tv[j] = a.T[g * K + j];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) add((int)w8[j], tv + j * K);
+            for (int kk = 0; kk < K; ++kk) {
+                if (columns.value) h[(state * K + kk) * bd + threadIdx.x] += t[kk];
+                else atomicAdd(&h[state * K + kk], t[kk]);
             }
-            s = s0 + ((s1 - s0) & ~(int64_t)7);
-        }
-        // the rest, four samples per thread in flight
-        for (int64_t q0 = s + threadIdx.x; q0 < s1; q0 += 4 * (int64_t)bd) {
-            int i[4];
-            AT tv[4][K];
+        };
+        constexpr int kF = 4;   // of the rest, samples per thread in flight
+        for (int ji = unit.y; ji < unit.z; ++ji) {
+            const cstate_t* st = a.cidxT + (int64_t)pb.class_inst[ji] * a.n_s;
+            int64_t s = s0;
+            if (vec) {
+                for (int64_t g = s0 + 8 * (int64_t)threadIdx.x; g + 8 <= s1; g += 8 * (int64_t)bd) {
+                    const uint4 sa = *(const uint4*)(st + g), sb = *(const uint4*)(st + g + 4);
+                    const uint32_t w8[8] = {sa.x, sa.y, sa.z, sa.w, sb.x, sb.y, sb.z, sb.w};
+                    AT tv[8 * K];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int64_t qs = min(q0 + j * (int64_t)bd, s1 - 1);
-                i[j] = (int)st[qs];
+                    for (int j = 0; j < 8 * K; ++j) tv[j] = a.T[g * K + j];
 #pragma unroll
-                for (int kk = 0; kk < K; ++kk) tv[j][kk] = a.T[qs * K + kk];
+                    for (int j = 0; j < 8; ++j) add((int)w8[j], tv + j * K);
+                }
+                s = s0 + ((s1 - s0) & ~(int64_t)7);
             }
+            for (int64_t q0 = s + threadIdx.x; q0 < s1; q0 += kF * (int64_t)bd) {
+                int i[kF];
+                AT tv[kF][K];
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (q0 + j * (int64_t)bd < s1) add(i[j], tv[j]);
+                for (int j = 0; j < kF; ++j) {
+                    const int64_t qs = min(q0 + j * (int64_t)bd, s1 - 1);
+                    i[j] = (int)st[qs];
+#pragma unroll
+                    for (int kk = 0; kk < K; ++kk) tv[j][kk] = a.T[qs * K + kk];
+                }
+#pragma unroll
+                for (int j = 0; j < kF; ++j)
+                    if (q0 + j * (int64_t)bd < s1) add(i[j], tv[j]);
+            }
         }
-    }
+    };
+    if (own) run(std::true_type());
+    else run(std::false_type());
     AT* tot = own ? h + (size_t)d * K * bd : h;   // the CTA's sums
     if (own) {
         __syncthreads();

@@ -196,22 +196,22 @@ struct CorrArgs {
     AT* corr_raw;           // [ncp][K] sum over samples of t_s per state (zeroed by the caller)
     const int4* units;      // cluster work units (class, first, end into class_inst)
     int cap;                // elements of the kernel's shared memory
+    double from[4];         // samples of a unit from which threads keep histograms, by sites
     const int* stop;
 };
 
 constexpr int kCorrCluster = 8;  // CTAs per correlator (one thread-block cluster)
-// Whether the correlator kernel's threads keep a histogram each: at most 64 values
-// (d states of K vectors; 131 KB per CTA), and samples enough to pay for
-// clearing and adding up 256 of them.  Atomics cost the more the fewer states a
-// warp's lanes share, so the line goes with d squared.  Whole FP64 products with
+// Samples of a work unit from which the correlator kernel's threads keep a
+// histogram each (d states of K vectors, at most 64 values: 131 KB per CTA).  They
+// have to pay for clearing and adding up 256 histograms of d values, at
+// fewer CTAs per SM the larger K; an atomic costs what its warp's lanes meet on,
+// 32 over the effective number of states eff (the inverse of the chance that two
+// samples agree, at the sector's mean occupations).  Whole FP64 products with
 // columns / atomics, half filling and quarter filling: 276 pairs, K = 1, 1,025
 // samples 86 / 70 and 83 / 76 us, 2,049 88 / 83 and 90 / 108, 4,097 95 / 107 and
 // 94 / 160; K = 2, 2,049 152 / 112 and 150 / 146, 6,145 181 / 190 and 175 / 214; 36
 // three-site correlators, 4,097 92 / 64 and 91 / 72, 12,289 120 / 96 and 106 / 114.
-__host__ __device__ inline bool corr_columns(int d, int K, int64_t samples) {
-    return d * K <= 64 && samples >= (int64_t)6 * d * d * K;
-}
-
+__host__ __device__ inline double corr_columns_from(int d, double eff, int K) { return 9.0 * d * eff * K; }
 // out = raw / n - Obar (Obar . V) + shift V of the passes with FP32 sums
 struct FinArgs {
     DevProblem pb;

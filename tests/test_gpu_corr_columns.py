@@ -15,7 +15,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n", [40, 95, 96, 767, 768, 1535, 1536, 3072, 24575, 24576])
+@pytest.mark.parametrize("n", [40, 143, 144, 1151, 1152, 2303, 2304, 4608, 36863, 36864])
 def test_products_at_the_line(n):
     wl = inputs.hubbard("c", 4, 2, 4, 4, "pair", seed=5, n_walkers=1)
     sites = [[0, 1], [2, 3], [4, 5], [1, 2, 6], [3, 4, 7], [0], [5]]
