@@ -151,12 +151,14 @@ struct PassArgs {
     const uint32_t* fulltab;  // [P] element e | a << 16 | b << 24 in row-major order of the pairs a < b
     const double* V;          // [K][nv]
     const double* invC;       // [ncp]
-    double* T;                // [n_s][K]
+    double* T;                // [n_s][ts], the pass's K vectors first
+    int ts;
     double* pf_partial;       // [gridDim][nimg][K]
     int nimg;                 // entries of an image: npf, or npf + ncp with the correlators (no shared blocks)
     const double* Obar;       // not null: obv_part[gridDim][K] = partial Obar . V
     double* obv_part;
-    double* clear;            // not null: [ncp][K] to be cleared
+    double* clear;            // not null: nclear values to be cleared
+    int64_t nclear;
     int ni;                   // images; pass_warps(K) / ni warps share one
     int bounds[pass_warps(1) + 1];   // first orbital p of each of an image's owners, then M
     const int* stop;
@@ -167,7 +169,8 @@ struct FinishArgs {
     double inv_n;             // 1 / n_s
     const double* part;       // [nblk][nimg][K] the pass's images
     int nblk, nimg;
-    const double* corr_raw;   // [ncp][K] correlator sums (nimg = npf)
+    const double* corr_raw;   // [ncp][cs] correlator sums, the K vectors' first (nimg = npf)
+    int cs;
     const double* invC;
     const double* lead_part;  // partials of Obar . V, or of the sum of E_L (gradient)
     int n_lead;

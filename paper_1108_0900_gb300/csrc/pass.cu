@@ -138,7 +138,7 @@ __device__ void pass_run(const PassArgs& a, int cta, int ncta, unsigned char* sm
         }
     }
     if (a.clear)
-        for (int64_t i = (int64_t)cta * blockDim.x + threadIdx.x; i < pb.ncp * K; i += (int64_t)ncta * blockDim.x)
+        for (int64_t i = (int64_t)cta * blockDim.x + threadIdx.x; i < a.nclear; i += (int64_t)ncta * blockDim.x)
             a.clear[i] = 0.0;
     __syncthreads();
     const ST* pf = (const ST*)a.s_pf;
@@ -203,12 +203,12 @@ __device__ void pass_run(const PassArgs& a, int cta, int ncta, unsigned char* sm
                 for (int kk = 0; kk < K; ++kk) {
                     const double t = warp_sum(A::value(sum[kk]) + tc[kk]);
                     if (lane == 0) {
-                        a.T[s * K + kk] = t;
+                        a.T[s * a.ts + kk] = t;
                         B.t[j][kk] = A::make(t);
                     }
                 }
             } else if (lane < K) {
-                B.t[j][lane] = A::make(a.T[s * K + lane]);
+                B.t[j][lane] = A::make(a.T[s * a.ts + lane]);
             }
         }
         if (owners > 1) __syncthreads();
@@ -247,7 +247,7 @@ __device__ void pass_run(const PassArgs& a, int cta, int ncta, unsigned char* sm
                 for (int c = own * 32 + lane; c < pb.ncorr; c += 32 * owners) {
                     double* y = (double*)(my + (npf + pb.corr_off[c] + a.s_cidx[(sb + j) * a.ncst + c]) * K);
 #pragma unroll
-                    for (int kk = 0; kk < K; ++kk) y[kk] += a.T[(sb + j) * K + kk];
+                    for (int kk = 0; kk < K; ++kk) y[kk] += a.T[(sb + j) * a.ts + kk];
                 }
             __syncwarp();   // the next sample's elements may meet these addresses in other lanes
         }
@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(256) k_sr_finish(FinishArgs a) {
         for (int64_t k = (int64_t)(blockIdx.x - nb1) * blockDim.x + threadIdx.x; k < pb.ncp; k += stride) {
             double raw[K];
 #pragma unroll
-            for (int kk = 0; kk < K; ++kk) raw[kk] = a.corr_raw[k * K + kk];
+            for (int kk = 0; kk < K; ++kk) raw[kk] = a.corr_raw[k * a.cs + kk];
             finish(k, raw);
         }
     }
