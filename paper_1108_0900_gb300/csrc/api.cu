@@ -54,7 +54,7 @@ struct vmc_ctx {
     std::set<std::pair<int, int>> unit_kinds;   // states and correlators of the histogram-scatter work units
     int max_csites = 0;          // sites of the largest correlator
     struct PassPlan {            // launch shape of a pass with FP64 sums (see plan_pass)
-        int ni = 0;              // images per CTA
+        int ni = 0, owners = 0;  // images per CTA, warps that share one
         int nimg = 0;            // entries of an image
         int64_t n_s = -1;        // of the samples that it is for (-1: not planned)
         size_t smem = 0;
@@ -1244,13 +1244,23 @@ extern "C" int vmc_logpsi_backward(vmc_handle h, const double* w, double* grad, 
 // streaming passes over the O store
 // ---------------------------------------------------------------------------
 // launch shape of a pass with FP64 sums over K vectors (gather) or for the
-// gradient (t_s given, K = 2): as many images per CTA as shared memory holds,
-// up to one per warp
+// gradient (t_s given, K = 2).  An owner's share of a sample should fill its
+// warp: the FP64 pipe and the issue slots take a warp with ten elements like one
+// with 32.  So an image has an owner per 64 elements, and there are as many images
+// as make 16 scattering warps (32 for one vector of many elements or the gradient,
+// 8 for four vectors of few) or fit.  FP64 products over 40,001 samples, pair
+// correlators, with every warp an owner and as many images as fit, and so: 4x4
+// lattice, 2 + 2 electrons, one vector 113 and 86 us, four 248 and 193; 8 + 8, one
+// 105 and 90; 6x6, 9 + 9, two 271 and 223, four 530 and 453; 18 + 18, one 213 and 204.
 static int plan_pass(vmc_ctx* h, int K, bool gather, vmc_ctx::PassPlan** out) {
     vmc_ctx::PassPlan& L = h->pass_plan[!gather ? 3 : K == 1 ? 0 : K == 2 ? 1 : 2];
     if (L.n_s != h->n_s) {
         auto smem = [&](int nimg, int ni) { return pass_smem(h->npf, nimg, h->P, K, gather, ni); };
-        int ni = pass_warps(K);
+        const int warps = pass_warps(K);
+        int share = 1;
+        while (share < 16 && 128 * share <= h->P) share *= 2;
+        const int active = K == 1 || !gather ? (share >= 4 ? 32 : 16) : K == 2 ? 16 : share >= 8 ? 16 : 8;
+        int ni = std::max(1, active / share);
         while (ni > 1 && smem(h->npf, ni) > h->smem_optin) ni /= 2;
         if (smem(h->npf, ni) > h->smem_optin) {
             set_err("pairing block does not fit in shared memory");
@@ -1258,14 +1268,20 @@ static int plan_pass(vmc_ctx* h, int K, bool gather, vmc_ctx::PassPlan** out) {
         }
         // no more images than the samples of a CTA pay for: an image is cleared
         // and added up once per element of the pairing block
-        const double per_cta = (double)h->n_s * h->P / h->nsm;
+        const double per_cta = (double)h->n_s * std::max(h->P, 256) / h->nsm;
         while (ni > 1 && (double)ni * h->npf > per_cta) ni /= 2;
         // correlator blocks of up to four pairing blocks, each one's own, enter the
         // images where these fit all the same: 4x4 lattice, pair correlators, 4,096
-        // samples, about 1 us more in the pass for a launch of 10.7 us
+        // samples, about 1 us more in the pass for a launch of 10.7 us.  Of few
+        // electrons fewer images will do; of many, half the images cost more than the
+        // launch (8x8, 28 + 28 electrons, 20,001 samples 278 against 259 us)
         const int64_t all = h->npf + h->ncp;
+        int nw = ni;
+        while (share <= 2 && nw > 1 && smem((int)all, nw) > h->smem_optin) nw /= 2;
         const bool with = h->n_class == h->ncorr && h->ncp > 0 && all <= 4 * (int64_t)h->npf &&
-                          smem((int)all, ni) <= h->smem_optin;
+                          smem((int)all, nw) <= h->smem_optin;
+        if (with) ni = nw;
+        L.owners = std::min(warps / ni, std::max(share, active / ni));
         L.nimg = with ? (int)all : h->npf;
         L.smem = smem(L.nimg, ni);
         L.ni = ni;
@@ -1288,6 +1304,7 @@ static void pass_args(const vmc_ctx* h, const vmc_ctx::PassPlan& L, int K, const
     a.ts = K;
     a.pf_partial = (double*)h->d_pfpart;
     a.ni = L.ni;
+    a.owners = L.owners;
     a.nimg = L.nimg;
     if (L.nimg == h->npf && h->ncp > 0) {
         a.clear = h->d_corrraw;
@@ -1296,7 +1313,7 @@ static void pass_args(const vmc_ctx* h, const vmc_ctx::PassPlan& L, int K, const
     a.stop = stop;
     // orbitals where an image's owners begin: equal shares of the expected number
     // of pairs (p, q > p) at the sector's mean occupations
-    const int owners = pass_warps(K) / L.ni;
+    const int owners = L.owners;
     const double fu = (double)h->nu / h->ns, fd = (double)h->nd / h->ns;
     double total = 0.0, above = (fu + fd) * h->ns, run = 0.0;
     std::vector<double> w(h->M);

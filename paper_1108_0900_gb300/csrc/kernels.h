@@ -159,7 +159,7 @@ struct PassArgs {
     double* obv_part;
     double* clear;            // not null: nclear values to be cleared
     int64_t nclear;
-    int ni;                   // images; pass_warps(K) / ni warps share one
+    int ni, owners;           // images, and the warps that share one (the rest have no part in the scatter)
     int bounds[pass_warps(1) + 1];   // first orbital p of each of an image's owners, then M
     const int* stop;
 };

@@ -7,10 +7,9 @@
 // elements by their smaller orbital p = occ[a] (boundaries of about equal
 // expected work), so two warps never touch one address, whatever samples they
 // are at: an update is a plain load, add and store, and the only
-// synchronisation is one barrier per tile between gather and scatter.  There
-// are as many images as shared memory holds (two at 128 spin orbitals, one
-// per warp on small lattices, where a warp keeps its sample for both halves
-// and needs no barrier).  The sums have a fixed order.  Small correlator blocks
+// synchronisation is one barrier per tile between gather and scatter.  How many
+// images and owners: plan_pass.  A warp without a part in the scatter gathers the
+// next tile meanwhile.  The sums have a fixed order.  Small correlator blocks
 // enter the images too (in FP64, a warp's lanes over the correlators); larger ones
 // are summed from the t_s by a kernel of their own.
 //
@@ -87,6 +86,26 @@ struct PairAcc {
     }
 };
 
+// Sums of K values over the warp, the k-th in the lanes from 32 k / K on: the first
+// log2 K steps halve the values that a lane carries on, so four sums are 6 FP64 adds
+// (16 cycles each, whatever the lanes do), not 20.
+template <int K>
+__device__ __forceinline__ double warp_sums(double (&v)[K]) {
+    int o = 16;
+#pragma unroll
+    for (int n = K; n > 1; n /= 2, o /= 2) {
+        const bool up = threadIdx.x & o;
+#pragma unroll
+        for (int i = 0; i < n / 2; ++i) {
+            const double give = up ? v[i] : v[i + n / 2], keep = up ? v[i + n / 2] : v[i];
+            v[i] = keep + __shfl_xor_sync(VMC_FULL_MASK, give, o);
+        }
+    }
+#pragma unroll
+    for (; o > 0; o /= 2) v[0] += __shfl_xor_sync(VMC_FULL_MASK, v[0], o);
+    return v[0];
+}
+
 constexpr int kU = 4, kUs = 2;   // elements per lane in flight, gather and scatter
 
 // shared memory of one tile buffer
@@ -103,7 +122,7 @@ __device__ void pass_run(const PassArgs& a, int cta, int ncta, unsigned char* sm
     using A = typename std::conditional<std::is_same<ST, float>::value, PairAcc, PlainAcc>::type;
     using E = typename A::Elem;
     const DevProblem& pb = a.pb;
-    const int npf = pb.npf, N = pb.N, P = pb.P, ni = a.ni, owners = NW / ni, nimg = a.nimg;
+    const int npf = pb.npf, N = pb.N, P = pb.P, ni = a.ni, owners = a.owners, nimg = a.nimg;
     E* img = (E*)smem;                                           // [ni][nimg][K]
     E* vpf = img + (size_t)ni * nimg * K;                        // [npf][K]
     TileBuf<E, K, NW>* buf = (TileBuf<E, K, NW>*)(vpf + (GATHER ? (size_t)npf * K : 0));   // [2]
@@ -143,9 +162,15 @@ __device__ void pass_run(const PassArgs& a, int cta, int ncta, unsigned char* sm
     __syncthreads();
     const ST* pf = (const ST*)a.s_pf;
     const int im = wid / owners, own = wid % owners;
-    E* my = img + (size_t)im * nimg * K;
+    E* my = img + (size_t)im * nimg * K;   // (im >= ni: no part in the scatter)
     const int64_t per = (a.n_s + ncta - 1) / ncta;
     const int64_t s0 = min(a.n_s, cta * per), s1 = min(a.n_s, s0 + per);
+    uint32_t below[4];   // the orbitals below the first one of owner `lane`, 32 to a word
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int b = a.bounds[min(lane, owners)] - 32 * k;
+        below[k] = b >= 32 ? ~0u : b <= 0 ? 0u : (1u << b) - 1u;
+    }
     int cur = 0;
     for (int64_t sb = s0; sb < s1; sb += kPassTile, cur ^= 1) {
         TileBuf<E, K, NW>& B = buf[cur];
@@ -153,21 +178,29 @@ __device__ void pass_run(const PassArgs& a, int cta, int ncta, unsigned char* sm
         // ---- gather: the warp's samples of the tile ------------------------
         for (int j = wid; j < n; j += NW) {
             const int64_t s = sb + j;
-            int o[2];
+            int o[2], ck[2];
+            double ic[2];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int i = lane + 32 * h;
+                if (GATHER) ck[h] = i < pb.ncorr ? (int)(pb.corr_off[i] + a.s_cidx[s * a.ncst + i]) : -1;
                 o[h] = i < N ? a.s_occ[s * a.Nst + i] : 255;
                 if (i < N) {
                     B.occ[j][i] = (uint8_t)o[h];
                     B.rb[j][i] = (int16_t)pf_row_base(pb.M, o[h]);
                 }
             }
-            for (int f = 0; f <= owners; ++f) {   // a = electrons below the owner's first orbital
-                const int a0 = __popc(__ballot_sync(VMC_FULL_MASK, o[0] < a.bounds[f])) +
-                               __popc(__ballot_sync(VMC_FULL_MASK, o[1] < a.bounds[f]));
-                if (lane == 0) B.start[j][f] = (uint16_t)(a0 * (2 * N - a0 - 1) / 2);
+            if (GATHER)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) ic[h] = ck[h] >= 0 ? a.invC[ck[h]] : 0.0;
+            int a0 = 0;   // electrons below the first orbital of owner `lane`
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t m = ((o[0] >> 5) == k ? 1u << (o[0] & 31) : 0u) | ((o[1] >> 5) == k ? 1u << (o[1] & 31) : 0u);
+                a0 += __popc(__reduce_or_sync(VMC_FULL_MASK, m) & below[k]);
             }
+            if (lane < owners) B.start[j][lane] = (uint16_t)(a0 * (2 * N - a0 - 1) / 2);
+            if (lane == 0) B.start[j][owners] = (uint16_t)P;
             __syncwarp();
             if (GATHER) {
                 E sum[K];
@@ -177,12 +210,17 @@ __device__ void pass_run(const PassArgs& a, int cta, int ncta, unsigned char* sm
                     sum[kk] = A::make(0.0);
                     tc[kk] = 0.0;
                 }
-                for (int c = lane; c < pb.ncorr; c += 32) {
+                for (int c = lane + 64; c < pb.ncorr; c += 32) {
                     const int64_t k = pb.corr_off[c] + a.s_cidx[s * a.ncst + c];
                     const double ic = a.invC[k];
 #pragma unroll
                     for (int kk = 0; kk < K; ++kk) tc[kk] += a.V[kk * pb.nv + k] * ic;
                 }
+                double cv[2][K];   // the first two correlators of the lane: loaded before the row, used after it
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int kk = 0; kk < K; ++kk) cv[h][kk] = ck[h] >= 0 ? a.V[kk * pb.nv + ck[h]] : 0.0;
                 const ST* row = pf + s * a.Pst;
                 for (int r0 = lane; r0 < P; r0 += 32 * kU) {
                     decltype(load_w(row)) w[kU];
@@ -200,21 +238,24 @@ __device__ void pass_run(const PassArgs& a, int cta, int ncta, unsigned char* sm
                             for (int kk = 0; kk < K; ++kk) A::add(sum[kk], w[u], vpf[pq[u] * K + kk]);
                 }
 #pragma unroll
-                for (int kk = 0; kk < K; ++kk) {
-                    const double t = warp_sum(A::value(sum[kk]) + tc[kk]);
-                    if (lane == 0) {
-                        a.T[s * a.ts + kk] = t;
-                        B.t[j][kk] = A::make(t);
-                    }
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int kk = 0; kk < K; ++kk) tc[kk] += cv[h][kk] * ic[h];
+#pragma unroll
+                for (int kk = 0; kk < K; ++kk) tc[kk] += A::value(sum[kk]);
+                const double t = warp_sums<K>(tc);
+                if ((lane & (32 / K - 1)) == 0) {
+                    const int kk = lane / (32 / K);
+                    a.T[s * a.ts + kk] = t;
+                    B.t[j][kk] = A::make(t);
                 }
             } else if (lane < K) {
                 B.t[j][lane] = A::make(a.T[s * a.ts + lane]);
             }
         }
-        if (owners > 1) __syncthreads();
-        else __syncwarp();
+        __syncthreads();
         // ---- scatter: the owner's share of the image's samples ---------------
-        for (int j = im; j < n; j += ni) {
+        for (int j = im < ni ? im : n; j < n; j += ni) {
             const ST* row = pf + (sb + j) * a.Pst;
             E t[K];
 #pragma unroll
