@@ -41,6 +41,8 @@ template <typename R> struct term_sum;
 template <> struct term_sum<double> {
     double s = 0.0;
     __device__ __forceinline__ void add(double x) { s += x; }
+    // x y, or nothing (x may be infinite or NaN then)
+    __device__ __forceinline__ void add_product(bool none, double x, double y) { s = fma(none ? 0.0 : x, y, s); }
     __device__ __forceinline__ double value() const { return s; }
 };
 template <> struct term_sum<float> {
@@ -50,6 +52,10 @@ template <> struct term_sum<float> {
         const float bx = __fsub_rn(s, hi);
         lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bx)), __fsub_rn(x, bx)));
         hi = s;
+    }
+    __device__ __forceinline__ void add_product(bool none, float x, float y) {
+        const float p = x * y;
+        add(none ? 0.f : p);
     }
     __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
@@ -359,7 +365,7 @@ __device__ __forceinline__ R coulomb_exchange(const DevProblem& pb, int p, int q
 // belong to electron b or hole y alone; a second move is then two 16-byte
 // shared loads, its correlator pair, its integral and a dozen multiply-adds.
 // Every lane keeps its second moves (b, y) in registers.  W sites per lane.
-template <typename R, int W>
+template <typename R, int W, bool FULL>
 __device__ __forceinline__ void ab_doubles_mixed(const DevProblem& pb, const AbLayout& L, R* tab, const R* X, int XS,
                                                  const uint8_t* occ, const int8_t* orb_pos, const uint8_t* emp,
                                                  const int8_t* eidx, uint64_t dn, term_sum<R>& sum) {
@@ -451,13 +457,14 @@ __device__ __forceinline__ void ab_doubles_mixed(const DevProblem& pb, const AbL
                 __syncwarp();
 #pragma unroll
                 for (int u = 0; u < kAbSlots; ++u) {
+                    if (!FULL && c0 + 32 * u >= nd * ed) break;   // the warp's slot is past the end
                     const Quad<R> B = ev[sb[u]], Y = ev[nd + sy[u]];
                     const R t1 = fma(Y.x, xab[u], c1[u]);
                     const R sv = fma(Y.x, omr, fma(fxa, c3[u], -fma(-fyb[u], B.x, Y.y)));
                     const R rpf = fma(-sv, xba[u], fma(gxa, t1, c2[u] * B.y));
                     const int t = min(c0 + 32 * u + lane, nd * ed - 1);
-                    const R term = hm[u] * rpf * (B.z * Y.z * t2[4 * t + word_int(B.w) + word_int(Y.w)]);
-                    sum.add(hm[u] == R(0) ? R(0) : term);   // a vanishing integral's ratio may overflow
+                    // (a vanishing integral's ratio may overflow)
+                    sum.add_product(hm[u] == R(0), hm[u] * rpf, B.z * Y.z * t2[4 * t + word_int(B.w) + word_int(Y.w)]);
                 }
             }
         }
@@ -469,7 +476,7 @@ __device__ __forceinline__ void ab_doubles_mixed(const DevProblem& pb, const AbL
 // lanes, one per hole, form the factor of the hole's toggle on top of the two
 // removed electrons.  Rows of integrals: (a x|b y) and, by the pair symmetry,
 // (a y|b x) = (b x|a y), so a load touches the few rows of the lanes' x.
-template <typename R>
+template <typename R, bool FULL>
 __device__ __forceinline__ void ab_doubles_same(const DevProblem& pb, const AbLayout& L, R* tab, const R* X, int XS,
                                                 const uint8_t* occ, const uint8_t* emp, int sp, term_sum<R>& sum) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -530,11 +537,11 @@ __device__ __forceinline__ void ab_doubles_same(const DevProblem& pb, const AbLa
             __syncwarp();
 #pragma unroll
             for (int u = 0; u < kAbPairSlots; ++u) {
+                if (!FULL && c0 + 32 * u >= npair) break;   // the warp's slot is past the end
                 const Quad<R> Vx = ev[sx[u]], Vy = ev[sy[u]];
                 const R rpf = double_ratio<R>(Vx.x, Vx.y, Vy.x, Vy.y, xab, xba, Vy.z, Vy.w, fyx[u], Vx.z, h[u]);
                 const R d = hm[u] - hx[u];
-                const R term = d * rpf * (er[sx[u]] * er[sy[u]] * gxy[u] * rab);
-                sum.add(d == R(0) ? R(0) : term);
+                sum.add_product(d == R(0), d * rpf, er[sx[u]] * er[sy[u]] * gxy[u] * rab);
             }
             b += nw;
             while (b >= na && a < na) {
@@ -545,7 +552,7 @@ __device__ __forceinline__ void ab_doubles_same(const DevProblem& pb, const AbLa
     }
 }
 
-template <typename R, int W>
+template <typename R, int W, bool FULL>
 __global__ void __launch_bounds__(kAbThreads, sizeof(R) == 4 ? 5 : 3) k_ab_energy(AbArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ double red[kAbThreads / 32];
@@ -688,10 +695,10 @@ __global__ void __launch_bounds__(kAbThreads, sizeof(R) == 4 ? 5 : 3) k_ab_energ
                     e1 += (double)(hm * G[ix * GS + ia] * r);
                 }
                 __syncthreads();
-                ab_doubles_same<R>(pb, L, tab, X, XS, occ, emp, sp, sum);
+                ab_doubles_same<R, FULL>(pb, L, tab, X, XS, occ, emp, sp, sum);
                 if (sp == 0) {
                     __syncwarp();
-                    ab_doubles_mixed<R, W>(pb, L, tab, X, XS, occ, orb_pos, emp, eidx, dn, sum);
+                    ab_doubles_mixed<R, W, FULL>(pb, L, tab, X, XS, occ, orb_pos, emp, eidx, dn, sum);
                 }
             }
         }
@@ -783,7 +790,15 @@ __global__ void __launch_bounds__(kAbThreads, sizeof(R) == 4 ? 5 : 3) k_ab_energ
 template <typename R>
 static cudaError_t launch_ab(const AbArgs& a, int threads, size_t smem, int nsm, cudaStream_t st) {
     // a lane takes W sites (mixed doubles) and W electrons (rows of G)
-    auto kern = a.pb.ns <= 32 && a.pb.N <= 32 ? k_ab_energy<R, 1> : k_ab_energy<R, 2>;
+    const bool one = a.pb.ns <= 32 && a.pb.N <= 32;
+    // slots past the end: a branch for each where there are many, or in FP64, whose
+    // pipe takes an empty slot like a full one (16 orbitals, 8 + 8 electrons, 8,192
+    // samples: FP32 895 us without and 847 with branches, FP64 1,633 and 1,042); none where
+    // every slot is needed (24 orbitals, 65,536 samples, FP32: 12.16 and 12.62 ms)
+    const int ed = a.pb.ns - a.pb.nd;
+    auto kern = one ? k_ab_energy<R, 1, false> : k_ab_energy<R, 2, false>;
+    if constexpr (sizeof(R) == 4)
+        if (a.pb.nd * ed > 32 * (kAbSlots - 1)) kern = one ? k_ab_energy<R, 1, true> : k_ab_energy<R, 2, true>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int per = 0;
