@@ -199,7 +199,7 @@ int vmc_get_walkers(vmc_handle h, uint8_t* occ, uint64_t* step, void* stream);
 int vmc_sample(vmc_handle h, int n_burn, uint64_t seed, void* stream);
 
 /* Health of the last vmc_sample (no counterpart in the paper).  Every chain
- * sums ln|Psi'/Psi| over its accepted moves (FP64 sum of its ratios); for the
+ * keeps ln|Psi| relative to its start (FP64 product of its accepted ratios); for the
  * stored samples j > 0 of walker w this running change is compared with the
  * change of ln|Psi| evaluated from scratch in FP64 (vmc_logpsi):
  *   drift = |(run_j - run_0) - (lnPsi_j - lnPsi_0)|,
@@ -231,8 +231,8 @@ int vmc_sample_batch(const vmc_handle* hs, int n, int n_burn, const uint64_t* se
 
 /* out[b] = (S_b + shift I) V[b] (Eq. 7 with the covariance term) for every
  * handle b < n, each over its own samples: one streaming launch reads every
- * handle's store (the generic per-sample pass; its CTAs are split among the
- * problems in proportion to their stored bytes), then each handle's
+ * handle's store (the pass with FP64 sums; its CTAs are split among the
+ * problems by their stored elements and samples), then each handle's
  * correlator sums and finish run.  V and out are host arrays of n device
  * pointers to FP64 vectors of the handle's n_v; store is VMC_STORE_FP64 or
  * VMC_STORE_FP32 (FP64 accumulation).  Synchronizes `stream`.  Errors:

@@ -12,7 +12,8 @@
 // G[x][a], G[x][j] = sum_k F[x][o_k] X[k][j]; of a double move double_ratio.
 //
 // Correlators of at most two sites (pairs): the correlator factor of any
-// excitation is a product of the per-sample tables of ab_tables, and what an
+// excitation is a product of the per-sample tables of ab_tables (where they hold:
+// TableRange), and what an
 // excitation does not share with its neighbours is a handful of shared loads,
 // its integrals and a dozen multiply-adds (ab_doubles_mixed, ab_doubles_same).
 //
@@ -21,13 +22,15 @@
 // SM holds five samples, 20 warps; one warp per sample inside the walkers'
 // kernel left 12 warps per SM beside its tables and overran the instruction
 // cache (24 ms).  24 orbitals, 12 + 12 electrons, 65,536 samples, FP32, with the
-// sampling (2.5 ms) and the gradient: 13.6 ms; 136 ms with each excitation's
+// sampling (2.5 ms) and the gradient: 12.2 ms; 136 ms with each excitation's
 // correlator factor evaluated by itself, 700 instructions per excitation.  CTAs
-// per SM: 4 14.1, 5 13.6, 6 14.0 ms.
+// per SM, at an earlier state of the kernel: 4 14.1, 5 13.6, 6 14.0 ms.
 //
-// The sums and ratios keep the order and the roundings that they have in the
-// positions' order of the walker: on nearly singular blocks E_L's FP32 rounding
-// grows with |X|, and two orders differ by 1e-5 of the gradient's norm there.
+// The products G and H and the pfaffian ratios keep the order and the roundings
+// that they have in the positions' order of the walker: on nearly singular blocks
+// E_L's FP32 rounding grows with |X|, and two orders differ by 1e-5 of the gradient's
+// norm there.  FP32: the diagonal is summed in FP64, every double excitation in an
+// FP32 pair.
 #include "ansatz.cuh"
 #include "common.cuh"
 #include "kernels.h"
@@ -202,7 +205,7 @@ __device__ __forceinline__ double int_word(double, int i) { return __hiloint2dou
 
 // Pfaffian ratio of the double move a -> x, b -> y (orbitals p1 -> x, p2 ->
 // y): the second replacement on the rank-2-updated inverse, written out in G,
-// X, F and H[y][x] = sum_j F[y][o_j] G[x][j].  ab_doubles evaluates the same
+// X, F and H[y][x] = sum_j F[y][o_j] G[x][j].  ab_doubles_mixed evaluates the same
 // operations with those of b or y alone taken out of the pair loop: on nearly
 // singular blocks terms of order |X|^2 cancel down to |X|, and the shorter
 // identity G G - G G + X (F - H) rounds differently there.
@@ -215,8 +218,11 @@ __device__ __forceinline__ R double_ratio(R gxa, R gxb, R gya, R gyb, R xab, R x
     return fma(-sy, xba, fma(gxa, t1, sc * yb));
 }
 
-constexpr int kAbSlots = 5;       // second moves per lane of the mixed double excitations
-constexpr int kAbPairSlots = 3;   // hole pairs per lane of those of one spin
+// Second moves per lane of the mixed double excitations, hole pairs per lane of those
+// of one spin: what 24 orbitals with 12 + 12 electrons need in one round of the
+// registers; smaller problems leave slots empty (launch_ab), larger ones take rounds.
+constexpr int kAbSlots = 5;
+constexpr int kAbPairSlots = 3;
 
 // The correlator factors of a sample's excitations for correlators of at most
 // two sites (the pair correlators of the ab initio ansatz), as tables over

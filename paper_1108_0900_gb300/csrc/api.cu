@@ -148,7 +148,10 @@ struct vmc_ctx {
     double* d_Obar[3] = {nullptr, nullptr, nullptr};
     float* d_Obar32[3] = {nullptr, nullptr, nullptr};   // FP32 copies for the inner solve
     int* d_status = nullptr;
-    bool status_live = false;   // a kernel that may set d_status was given it since the last read_status
+    // a kernel that may set d_status was given it since the last read_status.  Every
+    // entry that hands the word out reads it on its own stream before it returns,
+    // so no kernel that could still set it outlives a call that succeeded
+    bool status_live = false;
     // scratch
     void* d_T = nullptr;
     void* d_pfpart = nullptr;

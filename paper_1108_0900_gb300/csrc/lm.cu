@@ -44,7 +44,7 @@
 // 64 registers, eight samples per SM at 24 orbitals); FP64: the FP64 pipe.  24
 // orbitals, 12 + 12 electrons, 65,536 samples, FP32: 6.7 ms; one warp per sample
 // that divided out every correlator of every move and added it with an atomic
-// took 47.4 ms.  4x4 lattice, 2x2 correlators, 4,097 samples, FP64: 0.35 ms,
+// took 47.4 ms.  4x4 lattice, 2x2 correlators, 4,097 samples, FP64: 0.32 ms,
 // 0.57 before.  Threads x CTAs per SM by registers, FP32: 128 x 4 8.1, x 6 7.5,
 // x 8 6.7 ms; 256 threads 11.4, 8.6, 7.3 ms.
 #include <algorithm>

@@ -19,7 +19,7 @@
 // rounds at 56 electrons, not 56 rows of two half-empty ones), pairs (i, j) come
 // from a table, and 16 warps per SM hide the rest: it is 84 to 87 % busy.  16,384
 // samples at 56 electrons: inverse, E_L and O 4.1 ms (10.3 ms with the general
-// inverse of the walkers), the adjoint 3.7 ms (8.6), ln|Psi| 1.9 ms (5.7).
+// inverse of the walkers), the adjoint 3.6 ms (8.6), ln|Psi| 1.5 ms (5.7).
 #include "ansatz.cuh"
 #include "common.cuh"
 #include "kernels.h"

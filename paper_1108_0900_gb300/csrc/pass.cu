@@ -13,13 +13,14 @@
 // enter the images too (in FP64, a warp's lanes over the correlators); larger ones
 // are summed from the t_s by a kernel of their own.
 //
-// What bounds it: the FP64 store's pass the FP64 pipe (two FMAs per element, 72 %
+// What bounds it: the FP64 store's pass the FP64 pipe (two FMAs per element, 74 %
 // busy), the FP32 store's issue slots and shared-memory latency (32 warps).  8x8
-// lattice, 28 + 28 electrons: FP64 store, 65,536 samples 600 us (825 us with FP64
-// shared atomics), FP32 store, 131,072 samples 930 us (1,299 us with two shared
-// FP32 atomics per element).  Warps per CTA: 16 695 / 1,225 us, 32 600 / 930 us;
-// the FP32 store's gather in FP64 1,470 us (conversions fill the FP64 pipe);
-// scatter rounds of 4 elements per lane, skipped by the whole warp, 643 / 976 us.
+// lattice, 28 + 28 electrons: FP64 store, 65,536 samples 594 us (825 us with FP64
+// shared atomics), FP32 store, 131,072 samples 919 us (1,299 us with two shared
+// FP32 atomics per element).  At an earlier state (600 / 930 us), warps per CTA: 16
+// 695 / 1,225 us; the FP32 store's gather in FP64 1,470 us (conversions fill the FP64
+// pipe); scatter rounds of 4 elements per lane, skipped by the whole warp, 643 / 976
+// us.  Few electrons are bound by the latency of a tile's phases.
 //
 // Elements go in the row-major order of electron pairs a < b (fulltab), in
 // which an owner's share of a sample is one stretch; the tile's occupations
@@ -313,7 +314,7 @@ __device__ void pass_run(const PassArgs& a, int cta, int ncta, unsigned char* sm
 // other blocks the correlator sums that another kernel left in corr_raw.
 // A small product is its launches: with Obar . V, the clearing and the correlators
 // in the pass and everything after it here, 4x4 lattice, 4,096 samples, one vector
-// went from five kernels and a memset at 75 us a call to two at 47.
+// went from five kernels and a memset at 75 us a call to two at 46.
 template <int K, bool GRAD>
 __global__ void __launch_bounds__(256) k_sr_finish(FinishArgs a) {
     if (a.stop && *a.stop) return;

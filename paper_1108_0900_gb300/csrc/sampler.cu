@@ -14,10 +14,10 @@
 // Woodbury capacitance is r I, so
 //   X' = X + (c y^T - y c^T) / r,  c = X_{:,a},  y = X b + e_a.
 // The inverse is rebuilt from scratch (Gauss-Jordan, partial pivoting) at
-// the start of every call.  The chain also sums ln|ratio| of its accepted
-// moves (the logarithm in the chain's precision, the sum in FP64), the
-// running log-amplitude that a from-scratch evaluation of the stored samples
-// checks (vmc_sample_stats).
+// the start of every call.  The chain also multiplies up the magnitudes of its
+// accepted ratios in FP64 (LogProduct), whose logarithm at a stored sample is the
+// running log-amplitude that a from-scratch evaluation checks
+// (vmc_sample_stats).
 #include "ansatz.cuh"
 #include "common.cuh"
 #include "kernels.h"
